@@ -15,6 +15,7 @@
 //
 // Both kernels stream HBM: the export writes 24 B per pair (key and element), the apply
 // reads 24 B per pair (element and psi) plus two FP64 fused multiply-adds.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -220,8 +221,61 @@ __global__ void __launch_bounds__(32 * kExpWarps, 4) eloc_export_kernel(const __
     }
 }
 
-// One warp per sample: the P products summed lane-wise in FP64 (fixed lanes, fixed shuffle
-// tree: deterministic), then one complex division by psi(x).
+// E_loc of one sample from its sum of products, and the reports of a sample that has none.
+__device__ __forceinline__ void apply_finish(double re, double im, double2 p, double d, double2* __restrict__ eloc,
+                                             Counters* __restrict__ ctr) {
+    const double n2 = p.x * p.x + p.y * p.y;
+    double2 out;
+    if (n2 == 0.0 || !isfinite(d)) {
+        out.x = out.y = __longlong_as_double(0x7ff8000000000000LL);
+        atomicAdd(&ctr->bad, 1ULL);
+        if (n2 == 0.0) atomicOr(&ctr->flags, QC_FLAG_ZERO_PSI);
+        else {
+            atomicAdd(&ctr->invalid, 1ULL);
+            atomicOr(&ctr->flags, QC_FLAG_NELEC);
+        }
+    } else {
+        const double inv = 1.0 / n2;
+        out.x = d + (re * p.x + im * p.y) * inv;
+        out.y = (im * p.x - re * p.y) * inv;
+    }
+    *eloc = out;
+}
+
+// One lane's share of the products elems[j] psi[j], j = j0, j0 + step, ... < j1: kAppUnroll
+// independent partial sums (their loads in flight together), added in a fixed order.
+constexpr int kAppUnroll = 4;
+__device__ __forceinline__ double2 apply_products(const double* __restrict__ e, const double2* __restrict__ q,
+                                                  long long j0, long long j1, long long step) {
+    double re[kAppUnroll], im[kAppUnroll];
+#pragma unroll
+    for (int k = 0; k < kAppUnroll; ++k) re[k] = im[k] = 0.0;
+    long long j = j0;
+    for (; j + (kAppUnroll - 1) * step < j1; j += kAppUnroll * step) {
+        double h[kAppUnroll];
+        double2 v[kAppUnroll];
+#pragma unroll
+        for (int k = 0; k < kAppUnroll; ++k) {
+            h[k] = __ldcs(e + j + k * step);
+            v[k] = __ldcs(q + j + k * step);
+        }
+#pragma unroll
+        for (int k = 0; k < kAppUnroll; ++k) {
+            re[k] = fma(h[k], v[k].x, re[k]);
+            im[k] = fma(h[k], v[k].y, im[k]);
+        }
+    }
+    for (; j < j1; j += step) {
+        const double h = __ldcs(e + j);
+        const double2 v = __ldcs(q + j);
+        re[0] = fma(h, v.x, re[0]);
+        im[0] = fma(h, v.y, im[0]);
+    }
+    return make_double2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
+}
+
+// Many samples or short connected sets: one warp per sample.  The P products are summed
+// lane-wise in FP64 (fixed lanes, fixed shuffle tree: deterministic).
 __global__ void __launch_bounds__(256) eloc_apply_kernel(const double* __restrict__ elems,
                                                          const double* __restrict__ diag,
                                                          const double2* __restrict__ psi_conn,
@@ -232,48 +286,95 @@ __global__ void __launch_bounds__(256) eloc_apply_kernel(const double* __restric
     const long long warps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
     for (long long s = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); s < n_u;
          s += warps) {
-        const double* e = elems + s * P;
-        const double2* q = psi_conn + s * P;
-        // two independent partial sums per lane (j and j + 32 of each 64), added at the end
-        double re = 0.0, im = 0.0, re2 = 0.0, im2 = 0.0;
-        long long j = lane;
-        for (; j + 32 < P; j += 64) {
-            const double h0 = __ldcs(e + j), h1 = __ldcs(e + j + 32);
-            const double2 v0 = __ldcs(q + j), v1 = __ldcs(q + j + 32);
-            re = fma(h0, v0.x, re);
-            im = fma(h0, v0.y, im);
-            re2 = fma(h1, v1.x, re2);
-            im2 = fma(h1, v1.y, im2);
-        }
-        if (j < P) {
-            const double h0 = __ldcs(e + j);
-            const double2 v0 = __ldcs(q + j);
-            re = fma(h0, v0.x, re);
-            im = fma(h0, v0.y, im);
-        }
-        re = warp_sum(re + re2);
-        im = warp_sum(im + im2);
-        if (lane == 0) {
-            const double2 p = psi[s];
-            const double n2 = p.x * p.x + p.y * p.y;
-            const double d = diag[s];
-            double2 out;
-            if (n2 == 0.0 || !isfinite(d)) {
-                out.x = out.y = __longlong_as_double(0x7ff8000000000000LL);
-                atomicAdd(&ctr->bad, 1ULL);
-                if (n2 == 0.0) atomicOr(&ctr->flags, QC_FLAG_ZERO_PSI);
-                else {
-                    atomicAdd(&ctr->invalid, 1ULL);
-                    atomicOr(&ctr->flags, QC_FLAG_NELEC);
-                }
-            } else {
-                const double inv = 1.0 / n2;
-                out.x = d + (re * p.x + im * p.y) * inv;
-                out.y = (im * p.x - re * p.y) * inv;
-            }
-            eloc[s] = out;
-        }
+        const double2 t = apply_products(elems + s * P, psi_conn + s * P, lane, P, 32);
+        const double re = warp_sum(t.x), im = warp_sum(t.y);
+        if (lane == 0) apply_finish(re, im, psi[s], diag[s], eloc + s, ctr);
     }
+}
+
+// Long connected sets: 128 threads, or a cluster of R CTAs of 512, per sample.  The stream is
+// bound by HBM and, a close second, by the FP64 pipe (24 B and two fused multiply-adds per
+// pair), so what matters is that every SM has loads in flight whatever the number of samples:
+// a chunk of a large molecule is a few hundred samples of 10^6 pairs, and a warp per sample
+// left all but 200 warps of the chip idle (N=120, 200 samples, 5.7 GB: 11.1 ms; now 0.98 ms,
+// 5.9 TB/s).  Each CTA sums a contiguous share of the sample's pairs; the CTA sums are read
+// over distributed shared memory by the first CTA in rank order, so the result is
+// deterministic and needs no workspace.
+template <int T>
+__global__ void __launch_bounds__(T) eloc_apply_wide_kernel(const double* __restrict__ elems,
+                                                            const double* __restrict__ diag,
+                                                            const double2* __restrict__ psi_conn,
+                                                            const double2* __restrict__ psi, long long P,
+                                                            double2* __restrict__ eloc, Counters* __restrict__ ctr) {
+    __shared__ double2 warp_part[T / 32];
+    __shared__ double2 cta_part;
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const unsigned R = cl.num_blocks(), r = cl.block_rank();
+    const long long s = blockIdx.x / R;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double2 t = apply_products(elems + s * P, psi_conn + s * P, P * r / R + threadIdx.x, P * (r + 1) / R, T);
+    const double re = warp_sum(t.x), im = warp_sum(t.y);
+    if (lane == 0) warp_part[warp] = make_double2(re, im);
+    __syncthreads();
+    double sr = 0.0, si = 0.0;
+    if (warp == 0) {
+        const double2 v = lane < T / 32 ? warp_part[lane] : make_double2(0.0, 0.0);
+        sr = warp_sum(v.x);
+        si = warp_sum(v.y);
+        if (R > 1 && lane == 0) cta_part = make_double2(sr, si);
+    }
+    if (R > 1) {
+        cl.sync();
+        if (r == 0 && threadIdx.x == 0) {
+            for (unsigned k = 1; k < R; ++k) {
+                const double2 v = *cl.map_shared_rank(&cta_part, k);
+                sr += v.x;
+                si += v.y;
+            }
+        }
+        cl.sync();  // the other CTAs' sums stay in place until the first CTA has read them
+    }
+    if (r == 0 && threadIdx.x == 0) apply_finish(sr, si, psi[s], diag[s], eloc + s, ctr);
+}
+
+// Threads per sample: two full waves of the chip's threads over the samples; 32 (a warp), 128, or
+// R x 512 with R up to the portable cluster size.  With many samples a CTA's fixed cost (block
+// sum, launch) pays only for long sums (10,000 samples, P = 2,220: 140 us with a warp, 167 us with
+// 128 threads; P = 5,040: 277 against 311 us; P = 7,875: 381 against 361; P = 25,137: 1,102 against 983);
+// with few, idle SMs cost more (300 samples, P = 25,137: 270 us with a warp, 106 us).
+int apply_threads(long long n_u, long long P, int sm_count) {
+    const long long cap = n_u >= 8LL * sm_count ? P / 160 : P / 8;
+    const long long want = std::min(2LL * 2048 * sm_count / n_u, cap);
+    if (want <= 48) return 32;
+    if (want < 256 || (want < 512 && P < 32768)) return 128;
+    int t = 512;
+    while (t < 8 * 512 && want >= 2 * t) t *= 2;
+    return t;
+}
+
+template <int T>
+cudaError_t launch_apply_wide(const double* elems, const double* diag, const double2* conn, const double2* psi,
+                              long long n_u, long long P, double2* eloc, Counters* ctr, int R, cudaStream_t s) {
+    // a grid holds fewer than 2^31 blocks: longer chunks go out in several launches
+    const long long most = 0x7fffffffLL / R;
+    cudaError_t e = cudaSuccess;
+    for (long long lo = 0; lo < n_u && e == cudaSuccess; lo += most) {
+        const long long n = std::min(most, n_u - lo);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(static_cast<unsigned>(n * R));
+        cfg.blockDim = dim3(T);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = static_cast<unsigned>(R);
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, eloc_apply_wide_kernel<T>, elems + lo * P, diag + lo, conn + lo * P, psi + lo, P,
+                               eloc + lo, ctr);
+    }
+    return e;
 }
 
 qc_status ffail(qc_eloc* H, qc_status st, const std::string& m) {
@@ -336,11 +437,20 @@ extern "C" qc_status qc_eloc_apply(qc_eloc* H, const double* psi, const int64_t*
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(H->d_ctr, 0, sizeof(qc::Counters), s);
     if (e == cudaSuccess && n_u > 0) {
-        const long long blocks = std::min<long long>((n_u + 7) / 8, static_cast<long long>(H->sm_count) * 16);
-        qc::eloc_apply_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
-            elems, diag, reinterpret_cast<const double2*>(psi_conn), reinterpret_cast<const double2*>(psi), n_u,
-            H->sp.pairs, reinterpret_cast<double2*>(eloc_out), H->d_ctr);
-        e = cudaGetLastError();
+        const double2* conn = reinterpret_cast<const double2*>(psi_conn);
+        const double2* p2 = reinterpret_cast<const double2*>(psi);
+        double2* el = reinterpret_cast<double2*>(eloc_out);
+        const int t = qc::apply_threads(n_u, H->sp.pairs, H->sm_count);
+        if (t >= 512) {
+            e = qc::launch_apply_wide<512>(elems, diag, conn, p2, n_u, H->sp.pairs, el, H->d_ctr, t / 512, s);
+        } else if (t == 128) {
+            e = qc::launch_apply_wide<128>(elems, diag, conn, p2, n_u, H->sp.pairs, el, H->d_ctr, 1, s);
+        } else {
+            const long long blocks = std::min<long long>((n_u + 7) / 8, static_cast<long long>(H->sm_count) * 16);
+            qc::eloc_apply_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(elems, diag, conn, p2, n_u,
+                                                                              H->sp.pairs, el, H->d_ctr);
+            e = cudaGetLastError();
+        }
     }
     if (e == cudaSuccess) {
         qc::EvalParams ep{};
