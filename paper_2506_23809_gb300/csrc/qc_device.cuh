@@ -742,13 +742,14 @@ __device__ __forceinline__ void double_element(unsigned orbs, ulonglong2 px, con
 }
 
 // Per-sample set-up shared by both main kernels.  Returns false when x does not hold
-// na alpha and nb beta electrons below n_orb (then nothing is written to the lists).
+// na alpha and nb beta electrons below n_orb (then nothing is written to the lists).  The
+// diagonal is left out when with_diag is false.
 __device__ __forceinline__ bool sample_setup(const SysParams& sp, ulonglong2 x, int lane,
                                              unsigned char* wl,
                                              const unsigned long long* __restrict__ T64,
                                              unsigned long long& hx, double& ediag,
                                              unsigned long long& As, unsigned long long& Bs,
-                                             unsigned long long& hxa) {
+                                             unsigned long long& hxa, bool with_diag = true) {
     unsigned char* occA = wl;
     unsigned char* virA = wl + 64;
     unsigned char* occB = wl + 128;
@@ -790,6 +791,7 @@ __device__ __forceinline__ bool sample_setup(const SysParams& sp, ulonglong2 x, 
     As = A;
     Bs = B;
     __syncwarp();
+    if (!with_diag) return true;
     // diagonal: sum_p h_pp + 1/2 sum_{p,q occ} [(pp|qq) - d(sp,sq) (pq|qp)]  (FP64).  The
     // n_occ^2 ordered pairs of occupied spatial orbitals (positions 0 .. oa - 1 alpha, then
     // beta) are spread over the 32 lanes, one load and one add each: X holds the same-spin

@@ -29,8 +29,29 @@
 namespace qc {
 namespace {
 
-constexpr int kExpWarps = 8;
-constexpr int kPer = 2;  // double excitations per lane per step of the export (4 measured slower)
+// ------------------------------------------------------------------------------------
+// K8: export of the connected sets
+// ------------------------------------------------------------------------------------
+// The export writes 24 B per pair, so its floor is HBM's write rate; what bounds it below that
+// is the work per pair.  One CTA takes a contiguous range of one sample's output (a work item
+// from a device cursor).  For each double class the part of an excitation that its outer entry u
+// fixes and the part that its inner entry w fixes are each formed once per item, in shared
+// memory, as a record:
+//   u: the key with u's orbitals flipped, the mask of orbitals strictly between u's two, its
+//      share of the phase and of the integral indexes
+//   w: the key bits of w's orbitals, their positions, share of the phase, integral offset
+// A pair is then two key XORs, one or two integral loads, one subtraction for equal spins and
+// three phase bits: the pairs [i < j] .. [b < a] of the phase reduce to "is w's first (second)
+// orbital between u's two".  Consecutive pairs go to consecutive lanes, so keys and elements
+// leave in whole sectors, and the integrals are read with w's fastest index innermost
+// ((ai|jb); (jb|ia) and (ib|ja) for equal spins: the 8-fold symmetry of (pq|rs)), neighbouring
+// lanes in neighbouring words.  Before, every lane decoded its excitation from scratch (193 warp
+// instructions per 32 pairs, the FP64 pipe 59% busy with negations, gathers over strides of K^3).
+// N=52, 10,000 samples: 1.72 ms (3.5 TB/s); now 1.03 ms (5.9 TB/s; 48 registers and five CTAs of
+// 256 threads an SM; 61 registers and four: 1.09); N=120, 100 samples 2.67 -> 0.60 ms; N=104,
+// 70 electrons, 12 samples 1.22 -> 0.065 ms.
+constexpr long long kExpItemPairs = 10240;  // pairs of a work item (a single counts as export_single_weight)
+constexpr int kExpUTile = 256;  // outer entries whose records are in shared memory at a time
 
 struct ExportOut {
     ulonglong2* keys;   // [n_u * P] or null
@@ -38,186 +59,239 @@ struct ExportOut {
     double* diag;       // [n_u] or null
 };
 
-// Work item (sample s, part c of C): part c takes the singles when c = 0 and the outer
-// entries c, c + C, ... of each double class; items are handed out from a device cursor so
-// that the launch ends with little tail.
-template <int PREC>
-__global__ void __launch_bounds__(32 * kExpWarps, 4) eloc_export_kernel(const __grid_constant__ SysParams sp,
-                                                                     const ulonglong2* __restrict__ samples,
-                                                                     long long n_u,
-                                                                     const unsigned long long* __restrict__ Tg,
-                                                                     const ExportOut out, int C,
-                                                                     unsigned long long* __restrict__ cursor) {
+struct alignas(16) ExpU {
+    ulonglong2 key;            // x with u's orbitals flipped
+    unsigned long long between;  // spatial orbitals (of w's spin) strictly between u's two
+    unsigned d1;               // integral index share of (ai|bj), phase share in bit 31
+    unsigned d2;               // of (aj|bi) (equal spins)
+};
+
+// shared memory of an item: occupation lists, u records, w key bits, w words
+__host__ __device__ inline int exp_max_w(const SysParams& sp) {
+    int n = sp.nsb;
+    if (sp.npoa > 0 && sp.npva > n) n = sp.npva;
+    if (sp.npob > 0 && sp.npvb > n) n = sp.npvb;
+    return n;
+}
+constexpr size_t kExpOffList = kOffVar;
+constexpr size_t kExpOffU = kExpOffList + 256;
+constexpr size_t kExpOffW = kExpOffU + kExpUTile * sizeof(ExpU);
+inline size_t export_smem_bytes(const SysParams& sp) { return kExpOffW + static_cast<size_t>(exp_max_w(sp)) * (16 + 4); }
+
+__device__ __forceinline__ ulonglong2 key_bits(int p, int q) {
+    ulonglong2 k = make_ulonglong2(0ULL, 0ULL);
+    flip(k, p);
+    flip(k, q);
+    return k;
+}
+
+// One class of doubles over the output positions [lo, hi) of the class (the block's threads).
+// ab: an alpha-beta class (u an alpha single, w a beta single), else equal spins (u an occupied
+// pair, w an empty pair of spin `spin`).
+template <int PREC, int T, bool AB>
+__device__ __forceinline__ void export_doubles(const SysParams& sp, const ExportOut& out, ulonglong2 x, ulonglong2 px,
+                                               int spin, int n2, int lo, int hi, long long base, unsigned char* smem) {
+    const unsigned short* lut = reinterpret_cast<const unsigned short*>(smem + kOffLut);
+    const unsigned char* divA = smem + kOffDiv;
+    const unsigned char* divB = divA + 1024;
+    const unsigned char* wl = smem + kExpOffList;
+    const unsigned char* occ = wl + (AB ? 0 : 128 * spin);
+    const unsigned char* vir = wl + 64 + (AB ? 0 : 128 * spin);
+    ExpU* U = reinterpret_cast<ExpU*>(smem + kExpOffU);
+    ulonglong2* WK = reinterpret_cast<ulonglong2*>(smem + kExpOffW);
+    unsigned* WI = reinterpret_cast<unsigned*>(WK + exp_max_w(sp));
+    const int K = sp.K;
+    const unsigned K2 = static_cast<unsigned>(K) * K;
+    __syncthreads();  // the previous class's records are read no more
+    for (int w = threadIdx.x; w < n2; w += T) {
+        int k1, k2;  // w's spatial orbitals: (empty, occupied) beta or the empty pair a < b
+        unsigned off, par;
+        if (AB) {
+            const int jo = divB[w];
+            k2 = wl[128 + jo];
+            k1 = wl[192 + (w - jo * sp.vb)];
+            off = static_cast<unsigned>(k2 * K + k1);  // (ai|jb): kj K + kb
+            par = pbit(px, 2 * k2 + 1) ^ pbit(px, 2 * k1 + 1) ^ (k2 < k1 ? 1 : 0);
+            WK[w] = key_bits(2 * k2 + 1, 2 * k1 + 1);
+        } else {
+            const unsigned p = lut[w];
+            k1 = vir[p & 255u];
+            k2 = vir[p >> 8];
+            off = static_cast<unsigned>(k2) * K2 + k1;  // (jb|ia) and (ib|ja): kb K^2 + ka
+            par = pbit(px, 2 * k1 + spin) ^ pbit(px, 2 * k2 + spin);
+            WK[w] = key_bits(2 * k1 + spin, 2 * k2 + spin);
+        }
+        WI[w] = static_cast<unsigned>(k1) | (static_cast<unsigned>(k2) << 6) | (par << 12) | (off << 13);
+    }
+    const int u_end = (hi - 1) / n2 + 1;
+    const int sq = T / n2, sr = T - sq * n2;  // a step of the block in (u, w)
+    for (int ut = lo / n2; ut < u_end; ut += kExpUTile) {
+        const int nu = u_end - ut < kExpUTile ? u_end - ut : kExpUTile;
+        if (ut != lo / n2) __syncthreads();
+        for (int k = threadIdx.x; k < nu; k += T) {
+            const int u = ut + k;
+            ExpU r;
+            r.key = x;
+            int p, q;  // u's spatial orbitals
+            unsigned par;
+            if (AB) {
+                const int io = divA[u];
+                p = occ[io];
+                q = vir[u - io * sp.va];
+                flip(r.key, 2 * p);
+                flip(r.key, 2 * q);
+                par = pbit(px, 2 * p) ^ pbit(px, 2 * q) ^ (p < q ? 1 : 0);
+                // beta orbitals between the alpha orbitals 2p and 2q: spatial min .. max - 1
+                const int l = p < q ? p : q, h = p < q ? q : p;
+                r.between = (1ULL << h) - (1ULL << l);
+                r.d1 = (static_cast<unsigned>(q) * K + p) * K2;
+                r.d2 = 0u;
+            } else {
+                const unsigned pu = lut[u];
+                p = occ[pu & 255u];
+                q = occ[pu >> 8];
+                flip(r.key, 2 * p + spin);
+                flip(r.key, 2 * q + spin);
+                par = pbit(px, 2 * p + spin) ^ pbit(px, 2 * q + spin) ^ 1;  // [i < j] holds
+                r.between = (1ULL << q) - (1ULL << (p + 1));
+                r.d1 = static_cast<unsigned>(q) * K2 * K + static_cast<unsigned>(p) * K;  // (jb|ia)
+                r.d2 = static_cast<unsigned>(p) * K2 * K + static_cast<unsigned>(q) * K;  // (ib|ja)
+            }
+            r.d1 |= par << 31;
+            U[k] = r;
+        }
+        __syncthreads();
+        const int t_end = hi < (ut + nu) * n2 ? hi : (ut + nu) * n2;
+        int t = (lo > ut * n2 ? lo : ut * n2) + static_cast<int>(threadIdx.x);
+        int u = t / n2 - ut, w = t - (t / n2) * n2;
+        for (; t < t_end; t += T) {
+            const ExpU r = U[u];
+            const unsigned wi = WI[w];
+            if (out.elems) {
+                const unsigned off = wi >> 13, d = (r.d1 & 0x7fffffffu) + off;
+                const unsigned neg = (r.d1 >> 31) ^ (wi >> 12) ^ static_cast<unsigned>(r.between >> (wi & 63u)) ^
+                                     static_cast<unsigned>(r.between >> ((wi >> 6) & 63u));
+                double val;
+                if (PREC == QC_FP64) {
+                    double e = __ldg(sp.eri + QC_IX(d, QC_K4(sp), sp.err));
+                    if (!AB) e -= __ldg(sp.eri + QC_IX(r.d2 + off, QC_K4(sp), sp.err));
+                    val = with_sign(e, (neg & 1u) != 0u);
+                } else {
+                    float e = __ldg(sp.eri32 + QC_IX(d, QC_K4(sp), sp.err));
+                    if (!AB) e -= __ldg(sp.eri32 + QC_IX(r.d2 + off, QC_K4(sp), sp.err));
+                    val = static_cast<double>(with_sign(e, (neg & 1u) != 0u));
+                }
+                __stcs(out.elems + base + t, val);
+            }
+            if (out.keys) {
+                const ulonglong2 k = WK[w];
+                __stcs(out.keys + base + t, make_ulonglong2(r.key.x ^ k.x, r.key.y ^ k.y));
+            }
+            u += sq;
+            w += sr;
+            if (w >= n2) {
+                w -= n2;
+                ++u;
+            }
+        }
+    }
+}
+
+// A single's element sums 3 n_elec / 2 integrals: it weighs as much as a quarter as many doubles, and
+// items are cut by weight, so that a sample's singles spread over several (N=104, 70 electrons, 12
+// samples: 130 us when the first item of a sample held all its singles, 65 us so).
+__host__ __device__ inline long long export_single_weight(const SysParams& sp) {
+    const long long w = 3LL * (sp.oa + sp.ob) / 8;
+    return w > 1 ? w : 1;
+}
+
+// Output position of weight v of a sample's weighted order (singles w each, then doubles 1 each).
+__host__ __device__ inline long long export_position(const SysParams& sp, long long v) {
+    const long long w = export_single_weight(sp), n = sp.nsa + sp.nsb;
+    return v < n * w ? (v + w - 1) / w : n + (v - n * w);
+}
+
+// Work item (sample s, part c of C): weights [c Q, (c + 1) Q) of the sample's output.
+template <int PREC, int T>
+__global__ void __launch_bounds__(T, 1280 / T) eloc_export_kernel(const __grid_constant__ SysParams sp,
+                                                                  const ulonglong2* __restrict__ samples, long long n_u,
+                                                                  const unsigned long long* __restrict__ Tg,
+                                                                  const ExportOut out, long long C, long long Q,
+                                                                  unsigned long long* __restrict__ cursor) {
     extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned long long item;
+    __shared__ int valid;
     fill_cta_tables(sp, Tg, smem);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char* wl = smem + kOffVar + 256 * warp;
+    unsigned char* wl = smem + kExpOffList;
     const unsigned long long* T64 = reinterpret_cast<const unsigned long long*>(smem + kOffT);
     const long long P = sp.pairs;
     const unsigned long long items = static_cast<unsigned long long>(n_u) * C;
+    const double nan = __longlong_as_double(0x7ff8000000000000LL);
     while (true) {
-        unsigned long long it = 0;
-        if (lane == 0) it = atomicAdd(cursor, 1ULL);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= items) break;
-        const long long s = static_cast<long long>(it / C);
-        const int c = static_cast<int>(it - static_cast<unsigned long long>(s) * C);
-        const ulonglong2 x = samples[s];
-        unsigned long long hx, As, Bs, hxa;
-        double ediag;
-        const bool ok = sample_setup(sp, x, lane, wl, T64, hx, ediag, As, Bs, hxa);
-        __syncwarp();
-        const double nan = __longlong_as_double(0x7ff8000000000000LL);
-        if (lane == 0 && out.diag && c == 0) out.diag[s] = ok ? ediag : nan;
-        const ulonglong2 px = prefix_parity(x);
-        long long off = static_cast<long long>(s) * P;
-        const unsigned char* occA = wl;
-        const unsigned char* virA = wl + 64;
-        const unsigned char* occB = wl + 128;
-        const unsigned char* virB = wl + 192;
-        const unsigned short* lut = reinterpret_cast<const unsigned short*>(smem + kOffLut);
-        const unsigned char* divA = smem + kOffDiv;
-        const unsigned char* divB = divA + 1024;
-        const int K = sp.K;
-        for (int cls = 0; cls < 5; ++cls) {
-            const int n1 = cls < 2 ? 1 : cls == 2 ? sp.npoa : cls == 3 ? sp.npob : sp.nsa;
-            const int n2 = cls == 0 ? sp.nsa : cls == 1 ? sp.nsb : cls == 2 ? sp.npva : cls == 3 ? sp.npvb : sp.nsb;
-            // singles in part 0; the outer entries of the doubles interleaved over the parts
-            for (int u = cls < 2 ? (c == 0 ? 0 : n1) : c; u < n1; u += cls < 2 ? 1 : C) {
-                // the part of the excitation fixed by u (uniform across the warp): emptied
-                // orbital(s), their bits and their share of the phase and of the integral index
-                int i = 0, j = 0, a0 = 0;
-                ulonglong2 xu = x;
-                int paru = 0;
-                const int sp_ = cls == 3 ? 1 : 0;
-                if (ok && cls >= 2) {
-                    if (cls == 4) {
-                        const int io = divA[u];
-                        i = 2 * occA[io];
-                        a0 = 2 * virA[u - io * sp.va];
-                        flip(xu, i);
-                        flip(xu, a0);
-                        paru = pbit(px, i) ^ pbit(px, a0);
-                    } else {
-                        const unsigned pu = lut[u];
-                        const unsigned char* occ = cls == 2 ? occA : occB;
-                        i = 2 * occ[pu & 255u] + sp_;
-                        j = 2 * occ[pu >> 8] + sp_;
-                        flip(xu, i);
-                        flip(xu, j);
-                        paru = pbit(px, i) ^ pbit(px, j);
-                    }
-                }
-                if (!ok || cls < 2) {
-                    for (int w0 = 0; w0 < n2; w0 += 32) {
-                        const int w = w0 + lane;
-                        if (w >= n2) continue;
-                        const long long pos = off + static_cast<long long>(u) * n2 + w;
-                        if (!ok) {  // not a determinant of this system: no connected set
-                            if (out.keys) __stcs(out.keys + pos, make_ulonglong2(0ULL, 0ULL));
-                            if (out.elems) __stcs(out.elems + pos, nan);
-                            continue;
-                        }
-                        // singles: the general path (a small share of the pairs)
-                        const unsigned code = (static_cast<unsigned>(cls) << 24) | static_cast<unsigned>(w);
-                        const unsigned orbs = decode(code, sp, wl, smem, nullptr, nullptr);
-                        if (out.keys) {
-                            unsigned long long h;
-                            __stcs(out.keys + pos, excite(orbs, x, hx, T64, h));
-                        }
-                        if (out.elems) {
-                            double h64 = 0.0;
-                            float h32 = 0.f;
-                            bool sneg = false;
-                            single_element<PREC>(orbs, px, sp, wl, nullptr, h64, h32, sneg);
-                            __stcs(out.elems + pos, PREC == QC_FP64 ? h64 : static_cast<double>(h32));
-                        }
-                    }
-                    continue;
-                }
-                // doubles: kPer excitations per lane per step (w, w + 32, ...), every integral
-                // load issued before any is used
-                for (int w0 = 0; w0 < n2; w0 += 32 * kPer) {
-                    int aa[kPer], bb[kPer], jj[kPer];
-                    bool v[kPer];
-#pragma unroll
-                    for (int h = 0; h < kPer; ++h) {
-                        const int w = w0 + 32 * h + lane;
-                        v[h] = w < n2;
-                        const int ww = v[h] ? w : 0;
-                        if (cls == 4) {
-                            const int jo = divB[ww];
-                            aa[h] = a0;
-                            jj[h] = 2 * occB[jo] + 1;
-                            bb[h] = 2 * virB[ww - jo * sp.vb] + 1;
-                        } else {
-                            const unsigned pw = lut[ww];
-                            const unsigned char* vir = cls == 2 ? virA : virB;
-                            jj[h] = j;
-                            aa[h] = 2 * vir[pw & 255u] + sp_;
-                            bb[h] = 2 * vir[pw >> 8] + sp_;
-                        }
-                    }
-                    double e1[kPer], e2[kPer];
-                    float f1[kPer], f2[kPer];
-#pragma unroll
-                    for (int h = 0; h < kPer; ++h) {
-                        e1[h] = e2[h] = 0.0;
-                        f1[h] = f2[h] = 0.f;
-                    }
-                    if (out.elems) {
-#pragma unroll
-                        for (int h = 0; h < kPer; ++h) {
-                            if (!v[h]) continue;
-                            const int ki = i >> 1, ka = aa[h] >> 1, kj = jj[h] >> 1, kb = bb[h] >> 1;
-                            const size_t d = ((static_cast<size_t>(ka) * K + ki) * K + kb) * K + kj;  // (ai|bj)
-                            const size_t d2 = ((static_cast<size_t>(ka) * K + kj) * K + kb) * K + ki;  // (aj|bi)
-                            if (PREC == QC_FP64) {
-                                e1[h] = __ldg(sp.eri + d);
-                                if (cls != 4) e2[h] = __ldg(sp.eri + d2);
-                            } else {
-                                f1[h] = __ldg(sp.eri32 + d);
-                                if (cls != 4) f2[h] = __ldg(sp.eri32 + d2);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int h = 0; h < kPer; ++h) {
-                        if (!v[h]) continue;
-                        const long long pos = off + static_cast<long long>(u) * n2 + w0 + 32 * h + lane;
-                        ulonglong2 xp = xu;
-                        if (cls == 4) {
-                            flip(xp, jj[h]);
-                            flip(xp, bb[h]);
-                        } else {
-                            flip(xp, aa[h]);
-                            flip(xp, bb[h]);
-                        }
-                        if (out.keys) __stcs(out.keys + pos, xp);
-                        if (out.elems) {
-                            // <ab||ij> and its phase exactly as double_element forms them
-                            const int ii = i, ja = jj[h], a = aa[h], b = bb[h];
-                            const int par = (paru ^ (cls == 4 ? (pbit(px, ja) ^ pbit(px, b)) : (pbit(px, a) ^ pbit(px, b)))) +
-                                            (ii < ja) + (ii < b) + (ja < b) + (ii < a) + (ja < a) + (b < a);
-                            double val;
-                            if (PREC == QC_FP64) {
-                                double e = e1[h];
-                                if (cls != 4) e -= e2[h];
-                                val = (par & 1) ? -e : e;
-                            } else {
-                                float e = f1[h];
-                                if (cls != 4) e -= f2[h];
-                                val = static_cast<double>((par & 1) ? -e : e);
-                            }
-                            __stcs(out.elems + pos, val);
-                        }
-                    }
+        __syncthreads();  // the tables are there; the previous item's lists are read no more
+        if (threadIdx.x < 32) {
+            unsigned long long it = 0;
+            if (threadIdx.x == 0) it = atomicAdd(cursor, 1ULL);
+            it = __shfl_sync(QC_FULLMASK, it, 0);
+            if (it < items) {
+                const long long s = static_cast<long long>(it / C);
+                unsigned long long hx, As, Bs, hxa;
+                double ediag = 0.0;
+                const bool first = it == static_cast<unsigned long long>(s) * C && out.diag != nullptr;
+                const bool ok = sample_setup(sp, samples[s], threadIdx.x, wl, T64, hx, ediag, As, Bs, hxa, first);
+                if (threadIdx.x == 0) {
+                    if (first) out.diag[s] = ok ? ediag : nan;
+                    valid = ok ? 1 : 0;
                 }
             }
-            off += static_cast<long long>(n1) * n2;
+            if (threadIdx.x == 0) item = it;
         }
-        __syncwarp();
+        __syncthreads();
+        if (item >= items) break;
+        const long long s = static_cast<long long>(item / C);
+        const long long v0 = (static_cast<long long>(item) - s * C) * Q;
+        const long long p0 = export_position(sp, v0), p1 = export_position(sp, v0 + Q) < P ? export_position(sp, v0 + Q) : P;
+        const ulonglong2 x = samples[s];
+        const long long off = s * P;
+        if (!valid) {  // not a determinant of this system: no connected set
+            for (long long p = p0 + threadIdx.x; p < p1; p += T) {
+                if (out.keys) __stcs(out.keys + off + p, make_ulonglong2(0ULL, 0ULL));
+                if (out.elems) __stcs(out.elems + off + p, nan);
+            }
+            continue;
+        }
+        const ulonglong2 px = prefix_parity(x);
+        // singles: the general path (a small share of the pairs)
+        for (long long p = p0 + threadIdx.x; p < p1 && p < sp.nsa + sp.nsb; p += T) {
+            const unsigned code = p < sp.nsa ? static_cast<unsigned>(p)
+                                             : (1u << 24) | static_cast<unsigned>(p - sp.nsa);
+            const unsigned orbs = decode(code, sp, wl, smem, nullptr, nullptr);
+            if (out.keys) __stcs(out.keys + off + p, excited_key(orbs, x));
+            if (out.elems) {
+                double h64 = 0.0;
+                float h32 = 0.f;
+                bool sneg = false;
+                single_element<PREC>(orbs, px, sp, wl, nullptr, h64, h32, sneg);
+                __stcs(out.elems + off + p, PREC == QC_FP64 ? h64 : static_cast<double>(h32));
+            }
+        }
+        // doubles, class by class: the item's share of each (a class holds fewer than 2^31 pairs)
+        long long c0 = sp.nsa + sp.nsb;
+#pragma unroll
+        for (int cls = 2; cls < 5; ++cls) {
+            const int n2 = cls == 2 ? sp.npva : cls == 3 ? sp.npvb : sp.nsb;
+            const long long n = static_cast<long long>(cls == 2 ? sp.npoa : cls == 3 ? sp.npob : sp.nsa) * n2;
+            const long long a = p0 > c0 ? p0 - c0 : 0, b = p1 - c0 < n ? p1 - c0 : n;
+            if (a < b) {
+                if (cls == 4)
+                    export_doubles<PREC, T, true>(sp, out, x, px, 0, n2, static_cast<int>(a), static_cast<int>(b),
+                                               off + c0, smem);
+                else
+                    export_doubles<PREC, T, false>(sp, out, x, px, cls - 2, n2, static_cast<int>(a),
+                                                static_cast<int>(b), off + c0, smem);
+            }
+            c0 += n;
+        }
     }
 }
 
@@ -399,21 +473,35 @@ extern "C" qc_status qc_eloc_export(qc_eloc* H, const uint64_t* samples, int64_t
     if (n_u == 0 || (!keys_out && !elems_out && !diag_out)) return QC_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     qc::ExportOut out{reinterpret_cast<ulonglong2*>(keys_out), elems_out, diag_out};
-    const size_t smem = qc::kOffVar + 256 * qc::kExpWarps;
-    // parts per sample: about 4,096 pairs each, at most 8
-    const int C = static_cast<int>(std::max<long long>(1, std::min<long long>(8, H->sp.pairs / 4096)));
-    const long long items = n_u * C;
-    const long long blocks = std::min<long long>((items + qc::kExpWarps - 1) / qc::kExpWarps,
-                                                 static_cast<long long>(H->sm_count) * 4);
+    const size_t smem = qc::export_smem_bytes(H->sp);
+    using Kernel = void (*)(qc::SysParams, const ulonglong2*, long long, const unsigned long long*, qc::ExportOut,
+                            long long, long long, unsigned long long*);
+    const bool f64 = H->precision == QC_FP64;
+    // an item's fixed part (cursor, occupation lists, records) costs a small CTA less: 128 threads
+    // for short connected sets (P = 2,220, 20,000 samples: 437 us with 256, 328 with 128; P = 609: 108
+    // and 79; P = 25,137: 1,029 and 1,118)
+    const int T = H->sp.pairs < 8192 ? 128 : 256;
+    const Kernel f = T == 128 ? (f64 ? qc::eloc_export_kernel<QC_FP64, 128> : qc::eloc_export_kernel<QC_FP32_COMP, 128>)
+                              : (f64 ? qc::eloc_export_kernel<QC_FP64, 256> : qc::eloc_export_kernel<QC_FP32_COMP, 256>);
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, T, smem);
+    if (e != cudaSuccess || per_sm < 1)
+        return qc::ffail(H, QC_ERR_CUDA, std::string("export: ") + cudaGetErrorString(e));
+    // pairs per work item: about kExpItemPairs, fewer when that leaves the chip's CTAs short of work
+    const long long resident = static_cast<long long>(per_sm) * H->sm_count;
+    const long long V = H->sp.pairs + (qc::export_single_weight(H->sp) - 1) * (H->sp.nsa + H->sp.nsb);
+    long long C = std::max<long long>(1, (V + qc::kExpItemPairs / 2) / qc::kExpItemPairs);
+    while (n_u * C < 2 * resident && V / (2 * C) >= 1024) C *= 2;
+    const long long Q = (V + C - 1) / C;
+    const long long blocks = std::min<long long>(n_u * C, resident);
     unsigned long long* cursor = &H->d_ctr->next;  // the handle's counters are free between evaluations
-    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
+    e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return qc::ffail(H, QC_ERR_CUDA, std::string("export: ") + cudaGetErrorString(e));
-    if (H->precision == QC_FP64)
-        qc::eloc_export_kernel<QC_FP64><<<static_cast<unsigned>(blocks), 32 * qc::kExpWarps, smem, s>>>(
-            H->sp, reinterpret_cast<const ulonglong2*>(samples), n_u, H->d_T, out, C, cursor);
-    else
-        qc::eloc_export_kernel<QC_FP32_COMP><<<static_cast<unsigned>(blocks), 32 * qc::kExpWarps, smem, s>>>(
-            H->sp, reinterpret_cast<const ulonglong2*>(samples), n_u, H->d_T, out, C, cursor);
+    const ulonglong2* sk = reinterpret_cast<const ulonglong2*>(samples);
+    const unsigned grid = static_cast<unsigned>(blocks);
+    f<<<grid, T, smem, s>>>(H->sp, sk, n_u, H->d_T, out, C, Q, cursor);
     e = cudaGetLastError();
     if (e != cudaSuccess) return qc::ffail(H, QC_ERR_CUDA, std::string("export launch: ") + cudaGetErrorString(e));
     return QC_OK;
