@@ -283,8 +283,8 @@ qc_status qc_eloc_apply(qc_eloc* handle, const double* psi, const int64_t* count
  *              set (keys_out and counts_out are then not a table)
  *   work       device scratch of qc_dedup_workspace_bytes(n_raw) bytes, 256-byte aligned,
  *              not shared with a concurrent call
- * A stable radix sort over ceil(n_orb / 8) 8-bit digits, then run lengths; exact (integer
- * work), so the result is bit-identical to any correct sort.  Errors (QC_ERR_ARG,
+ * The distinct keys are counted in a hash table and sorted, or the whole stream is sorted and
+ * its runs counted; exact (integer work), so the result is bit-identical to any correct sort.  Errors (QC_ERR_ARG,
  * QC_ERR_CAPACITY for a short workspace, QC_ERR_CUDA) return synchronously; the message
  * is qc_eloc_last_error(NULL). */
 int64_t qc_dedup_workspace_bytes(int64_t n_raw);

@@ -3,18 +3,31 @@
 // multiplicities, the input that qc_eloc_eval takes.  The paper names the construction of
 // this lookup table as what limits scaling once the unique-sample count grows.
 //
-// A stable least-significant-digit radix sort over the n_orb significant bits (8-bit
-// digits, ceil(n_orb / 8) passes), then run lengths:
-//   per pass  KH hist:    every warp counts the digits of its tile of keys
-//             scan:       exclusive prefix over the (digit, tile) counts, digit-major, so
-//                         equal digits keep the order of their tiles
-//             KS scatter: every warp walks its tile in order and sends each key to its
-//                         digit's next slot (__match_any_sync ranks equal digits within
-//                         the 32 keys of a step, so the sort is stable)
-//   unique    KU flags:   head-of-run flags, per-block counts; scan; KE emit: the head
-//                         keys, their positions; KC counts: differences of positions.
-// Traffic per key: 16 B read (hist) + 16 B read + 16 B written (scatter) per pass, then
-// 16 B read, 24 B written.  Every step is bound by HBM bandwidth.
+// A sampler's stream repeats its keys many times, so the keys are counted before they are
+// sorted, and only the distinct ones are sorted:
+//   KA count    one pass over the raw stream into a hash table of the distinct keys (a slot
+//               holds the raw position of its key's first comer and a count).  Each CTA counts
+//               what it sees in a table of its own in shared memory first, so a key that makes
+//               up a sixth of the stream costs the chip 152 global atomics, not 10^6.
+//   KL list     the distinct keys, unsorted
+//   KT tiles    tiles of 2,048 keys sorted in shared memory
+//   KM merge    runs merged in pairs until one is left (the run lengths and the number of
+//               passes that do something follow the device's count of distinct keys)
+//   KE emit     the sorted keys with their counts, looked up in the hash table
+// A stream with too many distinct keys for the hash table (a probe sequence longer than
+// kProbeMax ends the counting), or a short one, is sorted whole instead by the same KT and KM,
+// and its runs counted:
+//   KH heads    heads of runs per tile; their prefix sum; KR runs: the head keys and their
+//               positions; KC: multiplicities as differences of positions
+// Every kernel of both ways is launched; the device's flag decides which of them do anything.
+//
+// Keys of up to 64 orbitals are sorted as one word.  Traffic: 16 B per raw key, then 16 (or 32)
+// B per distinct key and merge pass, in place of 48 B per raw key and 8-bit digit: N=52, 10^7 raw
+// keys of 10^5 distinct: 1.02 ms with a radix sort of the whole stream, now 0.20 ms (counting 78 us,
+// listing 10, tiles 16, six merges 48, the rest launches and the clearing); of 4*10^5 distinct
+// 1.05 -> 0.26; N=120 1.92 -> 0.22.  Sorted whole: 131,000 raw keys 0.36 -> 0.08 ms; 10^7 raw keys of
+// 5*10^6 distinct 1.15 -> 1.11 ms (0.14 of them the counting that ends early); N=120, 4*10^6 of
+// 3*10^6 distinct 1.22 -> 0.79.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,92 +38,494 @@
 
 namespace {
 
-constexpr int kTile = 2048;           // keys per warp tile (64 steps of 32)
-constexpr int kWarpsPerBlock = 8;
-constexpr int kBins = 256;
 constexpr int kScanBlock = 1024;      // threads of a scan block
 constexpr int kScanItems = 4;         // items per thread of a scan block
 constexpr int kScanSeg = kScanBlock * kScanItems;
 
+constexpr int kSortThreads = 256;
+constexpr int kSortItems = 8;
+constexpr int kTile = kSortThreads * kSortItems;  // keys of a tile
+// Shorter streams are sorted whole: the hash table's fixed cost (clearing and listing it) is more
+// than the merge passes it saves (131,072 raw keys: 84 us whole, 108 us counted).
+constexpr long long kCountMinRaw = 1 << 19;
+constexpr unsigned kMaxSlots = 1u << 21;    // hash table: 24 MB, L2-resident
+constexpr unsigned kProbeMax = 16;          // reached near 0.4 of the slots filled
+constexpr int kCountThreads = 1024;
+
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+struct Ctrl {
+    unsigned bad;    // a key had a bit >= n_orb
+    unsigned full;   // the hash table is full (or not used): sort the whole stream
+    unsigned m;      // distinct keys listed
+    unsigned runs;   // distinct keys of the whole stream, sorted (0: it was not)
+};
+
+// bufA and bufB: the sort's two buffers when the whole stream is sorted.  When its distinct keys are
+// counted, both are in bufA's space (its halves) and the hash table takes that of bufB and heads.
 struct Layout {
-    size_t bufA, bufB, heads, table, sums, flag, total;
+    size_t bufA, bufB, heads, sums, ctrl, total;
+    unsigned slots;  // hash slots (0: not used), 8 + 4 bytes each
 };
 
 Layout layout(long long n) {
-    const long long tiles = (n + kTile - 1) / kTile;
-    const long long table_n = static_cast<long long>(kBins) * std::max<long long>(tiles, 1);
-    const long long scan_n = std::max(table_n, n);  // the unique stage scans n flags
-    const long long segs = (scan_n + kScanSeg - 1) / kScanSeg;
+    const size_t k = static_cast<size_t>(std::max<long long>(n, 1));
     Layout L{};
     size_t off = 0;
-    L.bufA = off; off = align256(off + static_cast<size_t>(std::max<long long>(n, 1)) * 16);
-    L.bufB = off; off = align256(off + static_cast<size_t>(std::max<long long>(n, 1)) * 16);
-    L.heads = off; off = align256(off + static_cast<size_t>(n + 1) * 8);
-    L.table = off; off = align256(off + static_cast<size_t>(std::max(table_n, n)) * 4);
-    L.sums = off; off = align256(off + static_cast<size_t>(segs + 1) * 4 + 4096);
-    L.flag = off; off = align256(off + 16);
+    L.bufA = off; off = align256(off + k * 16);
+    L.bufB = off; off = align256(off + k * 16);
+    L.heads = off; off = align256(off + (k + 1) * 8);
+    L.sums = off; off = align256(off + (k / kTile + 2) * 4 + 4096);
+    L.ctrl = off; off = align256(off + sizeof(Ctrl));
     L.total = off;
+    if (n >= kCountMinRaw) {
+        L.slots = kMaxSlots;
+        while (L.slots > 2ULL * static_cast<unsigned long long>(n)) L.slots >>= 1;  // 12 B a slot, 24 B a raw key
+    }
     return L;
 }
 
-__device__ __forceinline__ unsigned digit_of(const ulonglong2 k, int pass) {
-    const int b = 8 * pass;
-    return b < 64 ? static_cast<unsigned>((k.x >> b) & 255u) : static_cast<unsigned>((k.y >> (b - 64)) & 255u);
+// A sort key: one word for up to 64 orbitals, else two.
+struct Key1 {
+    unsigned long long v;
+    __device__ static Key1 of(ulonglong2 k) { return Key1{k.x}; }
+    __device__ static Key1 max() { return Key1{~0ULL}; }
+    __device__ ulonglong2 wide() const { return make_ulonglong2(v, 0ULL); }
+    __device__ bool less(const Key1& o) const { return v < o.v; }
+    __device__ bool same(const Key1& o) const { return v == o.v; }
+    __device__ unsigned long long mix() const { return v; }
+};
+struct alignas(16) Key2 {
+    unsigned long long lo, hi;
+    __device__ static Key2 of(ulonglong2 k) { return Key2{k.x, k.y}; }
+    __device__ static Key2 max() { return Key2{~0ULL, ~0ULL}; }
+    __device__ ulonglong2 wide() const { return make_ulonglong2(lo, hi); }
+    __device__ bool less(const Key2& o) const { return hi < o.hi || (hi == o.hi && lo < o.lo); }
+    __device__ bool same(const Key2& o) const { return lo == o.lo && hi == o.hi; }
+    __device__ unsigned long long mix() const { return lo ^ (hi * 0x9E3779B97F4A7C15ULL); }
+};
+
+// Two multiply-xorshift rounds (the finalizer of splitmix64, Vigna).
+template <typename K>
+__device__ __forceinline__ unsigned long long key_hash(const K& k) {
+    unsigned long long z = k.mix();
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
+    return z ^ (z >> 31);
 }
 
-// KH: per-tile digit counts, table[d * tiles + t]; pass 0 also checks the unused bits
-__global__ void __launch_bounds__(256) dedup_hist_kernel(const ulonglong2* __restrict__ src, long long n, int pass,
-                                                         long long tiles, unsigned* __restrict__ table,
-                                                         ulonglong2 high_mask, unsigned* __restrict__ flag) {
-    __shared__ unsigned hist[kWarpsPerBlock][kBins];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int d = lane; d < kBins; d += 32) hist[warp][d] = 0u;
-    __syncwarp();
-    const long long t = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + warp;
-    if (t < tiles) {
-        const long long i0 = t * kTile;
-        const long long i1 = i0 + kTile < n ? i0 + kTile : n;
-        bool bad = false;
-        for (long long i = i0 + lane; i < i1; i += 32) {
-            const ulonglong2 k = src[i];
-            if (pass == 0) bad = bad || (k.x & high_mask.x) || (k.y & high_mask.y);
-            atomicAdd(&hist[warp][digit_of(k, pass)], 1u);
+// ------------------------------------------------------------------------------------
+// KA: counting
+// ------------------------------------------------------------------------------------
+// Add c to the count of key k (raw position i) in the global table.  A slot is written once, by
+// compare-and-swap: the high half of its key's hash and the raw position (plus one) of the key.
+// The raw stream does not change, so what a reader compares is always complete.
+template <typename K>
+__device__ __forceinline__ bool slot_holds(unsigned long long e, const ulonglong2* __restrict__ raw, const K& k,
+                                           unsigned long long h) {
+    return (e >> 32) == (h >> 32) && K::of(raw[static_cast<unsigned>(e) - 1u]).same(k);
+}
+template <typename K>
+__device__ __forceinline__ void count_global(const ulonglong2* __restrict__ raw, const K& k, unsigned i, unsigned c,
+                                             unsigned long long h, unsigned long long* slot, unsigned* count,
+                                             unsigned mask, Ctrl* ctrl) {
+    unsigned s = static_cast<unsigned>(h >> 13) & mask;
+    for (unsigned it = 0; it < kProbeMax; ++it) {
+        unsigned long long e = __ldcg(slot + s);
+        if (e == 0ULL) e = atomicCAS(slot + s, 0ULL, (h >> 32 << 32) | (i + 1u));
+        if (e == 0ULL || slot_holds(e, raw, k, h)) {
+            atomicAdd(count + s, c);
+            return;
         }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1u);
+        s = (s + 1u) & mask;
+    }
+    atomicOr(&ctrl->full, 1u);
+}
+
+// Shared-memory table of a CTA, in buckets of two slots: a slot's tag goes 0 (free) -> 1 (being
+// written) -> hash | 2; its key and raw position are valid once the tag is a hash.  A key that finds
+// neither slot its own goes to its warp's queue and is counted in the global table when 32 have
+// come together: a step in which some lanes walk L2 and the others wait costs the whole warp two
+// microseconds.  The bucket is read with one load and the common case (the key is there) has one
+// branch; claiming a free slot is a second step that most warps skip.  10^7 raw keys of 10^5
+// distinct: 206 us with four single-slot probes in a loop and no queue, 144 with the queue (269
+// instructions per 32 keys), 78 us so (aggregating equal slots of a warp with __match_any_sync: 90).
+template <typename K>
+struct CountTable {
+    static constexpr int slots = sizeof(K) == 8 ? 8192 : 4096;
+    static constexpr int queue = 64;  // per warp: up to 31 waiting and 32 new
+    static constexpr size_t bytes = slots * (sizeof(K) + 12) + kCountThreads / 32 * queue * 4;
+};
+
+template <typename K>
+__global__ void __launch_bounds__(kCountThreads, 1) dedup_count_kernel(const ulonglong2* __restrict__ raw, long long n,
+                                                                      ulonglong2 high, unsigned long long* slot,
+                                                                      unsigned* count, unsigned mask, Ctrl* ctrl) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    constexpr int S = CountTable<K>::slots;
+    K* keys = reinterpret_cast<K*>(sm);
+    unsigned* tag = reinterpret_cast<unsigned*>(sm + S * sizeof(K));
+    unsigned* cnt = tag + S;
+    unsigned* pos = cnt + S;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned* queue = pos + S + warp * CountTable<K>::queue;
+    for (int t = threadIdx.x; t < S; t += kCountThreads) tag[t] = cnt[t] = 0u;
+    __syncthreads();
+    bool bad = false;
+    int qn = 0;
+    auto flush = [&](int m) {  // the first m queued raw positions to the global table
+        if (lane < m) {
+            const unsigned i = queue[lane];
+            const K k = K::of(raw[i]);
+            count_global(raw, k, i, 1u, key_hash(k), slot, count, mask, ctrl);
+        }
         __syncwarp();
-        for (int d = lane; d < kBins; d += 32) table[static_cast<long long>(d) * tiles + t] = hist[warp][d];
+        const unsigned rest = lane < qn - m ? queue[m + lane] : 0u;
+        __syncwarp();
+        if (lane < qn - m) queue[lane] = rest;
+        __syncwarp();
+        qn -= m;
+    };
+    constexpr int kLoads = 4;  // raw keys in flight per thread
+    const long long step = static_cast<long long>(gridDim.x) * kCountThreads * kLoads;
+    for (long long b = (static_cast<long long>(blockIdx.x) * kCountThreads + 32 * warp) * kLoads; b < n; b += step) {
+        ulonglong2 r[kLoads];
+#pragma unroll
+        for (int l = 0; l < kLoads; ++l)
+            if (b + 32 * l + lane < n) r[l] = __ldg(raw + b + 32 * l + lane);
+        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile unsigned*>(&ctrl->full) != 0u)) break;
+#pragma unroll
+        for (int l = 0; l < kLoads; ++l) {
+            const long long i = b + 32 * l + lane;
+            bool miss = i < n;
+            bad = bad || (miss && ((r[l].x & high.x) != 0ULL || (r[l].y & high.y) != 0ULL));
+            const K k = K::of(r[l]);
+            const unsigned long long h = key_hash(k);
+            const unsigned mine = static_cast<unsigned>(h >> 32) | 2u;
+            const unsigned s0 = static_cast<unsigned>(h) & (S - 2);
+            const volatile unsigned* vt = tag + s0;
+            const unsigned t0 = vt[0], t1 = vt[1];
+            __threadfence_block();
+            if (miss && (t0 == mine || t1 == mine)) {
+                const unsigned s = t0 == mine ? s0 : s0 + 1u;
+                if (keys[s].same(k)) {
+                    atomicAdd(cnt + s, 1u);
+                    miss = false;
+                }
+            }
+            if (__any_sync(0xffffffffu, miss && (t0 == 0u || t1 == 0u))) {
+                if (miss && (t0 == 0u || t1 == 0u)) {
+                    const unsigned s = t0 == 0u ? s0 : s0 + 1u;
+                    if (atomicCAS(tag + s, 0u, 1u) == 0u) {
+                        keys[s] = k;
+                        pos[s] = static_cast<unsigned>(i);
+                        atomicAdd(cnt + s, 1u);
+                        __threadfence_block();
+                        *reinterpret_cast<volatile unsigned*>(tag + s) = mine;
+                        miss = false;
+                    }
+                }
+                __syncwarp();
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, miss);
+            if (miss) queue[qn + __popc(m & ((1u << lane) - 1u))] = static_cast<unsigned>(i);
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) flush(32);
+        }
+    }
+    if (qn > 0) flush(qn);
+    if (bad) atomicOr(&ctrl->bad, 1u);
+    __syncthreads();
+    for (int t = threadIdx.x; t < S; t += kCountThreads)
+        if (tag[t] >= 2u)
+            count_global(raw, keys[t], pos[t], cnt[t], key_hash(keys[t]), slot, count, mask, ctrl);
+}
+
+// KL: the distinct keys into `list`, in any order (they are sorted next and are distinct).  (Listing
+// a key where it claims its slot costs the count an atomic on one address per distinct key: 158 ->
+// 297 us at 4*10^5.)
+constexpr int kListSlots = 4;  // slots a thread
+template <typename K>
+__global__ void __launch_bounds__(1024) dedup_list_kernel(const ulonglong2* __restrict__ raw,
+                                                          const unsigned long long* __restrict__ slot,
+                                                          K* __restrict__ list, Ctrl* ctrl) {
+    __shared__ unsigned warp_n[32];
+    __shared__ unsigned base;
+    if (ctrl->full != 0u) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long e[kListSlots];
+    unsigned have[kListSlots], before[kListSlots], n = 0;
+#pragma unroll
+    for (int t = 0; t < kListSlots; ++t) e[t] = __ldcg(slot + (blockIdx.x * kListSlots + t) * 1024u + threadIdx.x);
+#pragma unroll
+    for (int t = 0; t < kListSlots; ++t) {
+        have[t] = __ballot_sync(0xffffffffu, e[t] != 0ULL);
+        before[t] = n;
+        n += __popc(have[t]);
+    }
+    if (lane == 0) warp_n[warp] = n;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned v = warp_n[lane];
+        unsigned x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        warp_n[lane] = x - v;
+        if (lane == 31) base = x != 0u ? atomicAdd(&ctrl->m, x) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kListSlots; ++t)
+        if (e[t] != 0ULL)
+            list[base + warp_n[warp] + before[t] + __popc(have[t] & ((1u << lane) - 1u))] =
+                K::of(raw[static_cast<unsigned>(e[t]) - 1u]);
+}
+
+// Whether the whole stream is sorted: the hash table is not used or filled up, or holds more keys
+// than half of bufA does.
+template <typename K>
+__device__ __forceinline__ bool sort_whole(const Ctrl* ctrl, long long n) {
+    return ctrl->full != 0u || static_cast<long long>(ctrl->m) * static_cast<long long>(sizeof(K)) > 8 * n;
+}
+
+// ------------------------------------------------------------------------------------
+// KT, KM: sort
+// ------------------------------------------------------------------------------------
+// A tile in shared memory: one key of padding after eight, so that threads reading or writing
+// eight consecutive keys each hit different banks.
+template <typename K>
+struct Tile {
+    K* sh;
+    int at;
+    __device__ K& operator[](int i) const { return sh[at + i + ((at + i) >> 3)]; }
+};
+constexpr int kTilePadded = kTile + kTile / 8;
+
+// Keys a[0, na) before output position d of the merge of a and b (ties from a): the smallest i
+// with a[i] > b[d - 1 - i], by bisection.
+template <typename K>
+__device__ __forceinline__ int merge_split(Tile<K> a, int na, Tile<K> b, int nb, int d) {
+    int lo = d > nb ? d - nb : 0, hi = d < na ? d : na;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (b[d - 1 - mid].less(a[mid])) hi = mid; else lo = mid + 1;
+    }
+    return lo;
+}
+
+// kSortItems outputs of the merge of a[i, na) and b[j, nb) into registers.
+template <typename K>
+__device__ __forceinline__ void merge_items(Tile<K> a, int i, int na, Tile<K> b, int j, int nb, K (&out)[kSortItems]) {
+    K ka = i < na ? a[i] : K::max(), kb = j < nb ? b[j] : K::max();
+#pragma unroll
+    for (int t = 0; t < kSortItems; ++t) {
+        const bool from_b = i >= na || (j < nb && kb.less(ka));
+        out[t] = from_b ? kb : ka;
+        if (from_b) {
+            ++j;
+            kb = j < nb ? b[j] : K::max();
+        } else {
+            ++i;
+            ka = i < na ? a[i] : K::max();
+        }
     }
 }
 
-// KS: stable scatter of each tile in index order
-__global__ void __launch_bounds__(256) dedup_scatter_kernel(const ulonglong2* __restrict__ src,
-                                                            ulonglong2* __restrict__ dst, long long n, int pass,
-                                                            long long tiles, const unsigned* __restrict__ offs) {
-    __shared__ unsigned run[kWarpsPerBlock][kBins];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long t = static_cast<long long>(blockIdx.x) * kWarpsPerBlock + warp;
-    if (t >= tiles) return;  // warp-uniform; no block-wide barrier below
-    for (int d = lane; d < kBins; d += 32) run[warp][d] = offs[static_cast<long long>(d) * tiles + t];
-    __syncwarp();
-    const unsigned lt = (1u << lane) - 1u;
-    const long long i0 = t * kTile;
-    const long long i1 = i0 + kTile < n ? i0 + kTile : n;
-    for (long long b = i0; b < i1; b += 32) {
-        const long long i = b + lane;
-        const bool v = i < i1;
-        const unsigned active = __ballot_sync(0xffffffffu, v);
-        if (v) {
-            const ulonglong2 k = src[i];
-            const unsigned d = digit_of(k, pass);
-            const unsigned same = __match_any_sync(active, d);
-            const unsigned base = run[warp][d];
-            dst[base + __popc(same & lt)] = k;
-            __syncwarp(active);
-            if ((same & lt) == 0u) run[warp][d] = base + __popc(same);  // the lowest lane of the group
+// The block's keys from registers (8 consecutive ones a thread) to global memory, coalesced.
+template <typename K>
+__device__ __forceinline__ void store_tile(Tile<K> sh, const K (&v)[kSortItems], K* __restrict__ out, long long at, int n) {
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kSortItems; ++t) sh[threadIdx.x * kSortItems + t] = v[t];
+    __syncthreads();
+    for (int t = threadIdx.x; t < n; t += kSortThreads) out[at + t] = sh[t];
+}
+
+// KT: tiles of kTile keys of the list (or, whole, of the raw stream) sorted into `out`: eight
+// keys a thread by an odd-even network, then merges of 8, 16, .. 1,024 keys in shared memory.
+// `list` may be `out`: a tile is read whole before it is written.
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) dedup_tile_kernel(const ulonglong2* __restrict__ raw, long long n,
+                                                                  const K* list, K* out, ulonglong2 high, Ctrl* ctrl) {
+    __shared__ K tile[kTilePadded];
+    const Tile<K> sh{tile, 0};
+    const bool whole = sort_whole<K>(ctrl, n);
+    const long long m = whole ? n : static_cast<long long>(ctrl->m);
+    bool bad = false;
+    for (long long at = static_cast<long long>(blockIdx.x) * kTile; at < m;
+         at += static_cast<long long>(gridDim.x) * kTile) {
+        const int have = m - at < kTile ? static_cast<int>(m - at) : kTile;
+        __syncthreads();
+        for (int t = threadIdx.x; t < kTile; t += kSortThreads) {
+            K k = K::max();  // past the end: the largest key stays there
+            if (t < have) {
+                if (whole) {
+                    const ulonglong2 r = raw[at + t];
+                    bad = bad || (r.x & high.x) != 0ULL || (r.y & high.y) != 0ULL;
+                    k = K::of(r);
+                } else {
+                    k = list[at + t];
+                }
+            }
+            sh[t] = k;
         }
-        __syncwarp();
+        __syncthreads();
+        K v[kSortItems];
+#pragma unroll
+        for (int t = 0; t < kSortItems; ++t) v[t] = sh[threadIdx.x * kSortItems + t];
+#pragma unroll
+        for (int round = 0; round < kSortItems; ++round)
+#pragma unroll
+            for (int t = round & 1; t + 1 < kSortItems; t += 2)
+                if (v[t + 1].less(v[t])) {
+                    const K x = v[t];
+                    v[t] = v[t + 1];
+                    v[t + 1] = x;
+                }
+        for (int run = kSortItems; run < kTile; run *= 2) {
+            __syncthreads();
+#pragma unroll
+            for (int t = 0; t < kSortItems; ++t) sh[threadIdx.x * kSortItems + t] = v[t];
+            __syncthreads();
+            const int p = threadIdx.x * kSortItems, a0 = p / (2 * run) * (2 * run), d = p - a0;
+            const Tile<K> a{tile, a0}, b{tile, a0 + run};
+            const int i = merge_split(a, run, b, run, d);
+            merge_items(a, i, run, b, d - i, run, v);
+        }
+        store_tile(sh, v, out, at, have);
+    }
+    if (bad) atomicOr(&ctrl->bad, 1u);
+}
+
+// The split of output position d between the runs a[0, na) and b[0, nb) in global memory, by the
+// 32 lanes of a warp: each step cuts the range to a 33rd, so a run of 10^6 keys takes four
+// dependent loads instead of twenty.
+template <typename K>
+__device__ __forceinline__ long long merge_split_warp(const K* __restrict__ a, long long na, const K* __restrict__ b,
+                                                      long long nb, long long d, int lane) {
+    long long lo = d > nb ? d - nb : 0, hi = d < na ? d : na;  // the answer lies in [lo, hi]
+    while (lo < hi) {
+        const long long len = hi - lo;
+        // lane's probe in [lo, hi): ascending with the lane
+        const long long mid = lo + (len < 32 ? (lane < len ? lane : len - 1) : len * (lane + 1) / 33);
+        const bool after = !b[d - 1 - mid].less(a[mid]);  // the answer is beyond mid
+        const unsigned m = __ballot_sync(0xffffffffu, after);
+        // probes are ascending and `after` is true up to the answer: count the leading ones
+        const int c = m == 0xffffffffu ? 32 : __ffs(~m) - 1;
+        const long long below = __shfl_sync(0xffffffffu, mid, c > 0 ? c - 1 : 0);
+        const long long above = __shfl_sync(0xffffffffu, mid, c < 32 ? c : 31);
+        if (c > 0) lo = below + 1;
+        if (c < 32) hi = above;
+    }
+    return lo;
+}
+
+// KM: one merge pass: runs of `run` keys in pairs, from A to the other buffer (B, or for the listed
+// keys half) or, odd, back; kTile outputs a block and step.  Nothing is left to do once a run
+// holds every key.
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) dedup_merge_kernel(K* A, K* B, K* half, bool odd, long long n,
+                                                                   long long run, const Ctrl* ctrl) {
+    __shared__ K tile[kTilePadded];
+    __shared__ long long split[2];
+    const Tile<K> sh{tile, 0};
+    const bool whole = sort_whole<K>(ctrl, n);
+    const long long m = whole ? n : static_cast<long long>(ctrl->m);
+    if (run >= m) return;
+    K* other = whole ? B : half;
+    const K* in = odd ? other : A;
+    K* out = odd ? A : other;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (long long at = static_cast<long long>(blockIdx.x) * kTile; at < m;
+         at += static_cast<long long>(gridDim.x) * kTile) {
+        const long long a0 = at / (2 * run) * (2 * run);
+        const long long na = m - a0 < run ? m - a0 : run, nb = m - a0 - na < run ? m - a0 - na : run;
+        const long long d0 = at - a0, d1 = d0 + kTile < na + nb ? d0 + kTile : na + nb;
+        const K* a = in + a0;
+        const K* b = a + na;
+        if (warp < 2) {
+            const long long i = merge_split_warp(a, na, b, nb, warp == 0 ? d0 : d1, lane);
+            if (lane == 0) split[warp] = i;
+        }
+        __syncthreads();
+        const long long i0 = split[0], i1 = split[1], j0 = d0 - i0;
+        const int ca = static_cast<int>(i1 - i0), c = static_cast<int>(d1 - d0), cb = c - ca;
+        for (int t = threadIdx.x; t < c; t += kSortThreads) sh[t] = t < ca ? a[i0 + t] : b[j0 + (t - ca)];
+        __syncthreads();
+        const int d = static_cast<int>(threadIdx.x) * kSortItems < c ? static_cast<int>(threadIdx.x) * kSortItems : c;
+        const Tile<K> sb{tile, ca};
+        const int i = merge_split(sh, ca, sb, cb, d);
+        K v[kSortItems];
+        merge_items(sh, i, ca, sb, d - i, cb, v);
+        store_tile(sh, v, out, at, c);
+        __syncthreads();
+    }
+}
+
+// The buffer that holds the sorted keys: KT leaves them in A, every merge pass that did something
+// swaps the two.
+template <typename K>
+__device__ __forceinline__ const K* sorted_in(const K* A, const K* B, long long m) {
+    int passes = 0;
+    for (long long run = kTile; run < m; run *= 2) ++passes;
+    return (passes & 1) ? B : A;
+}
+
+// KE: the distinct keys with their counts.
+template <typename K>
+__global__ void __launch_bounds__(256) dedup_emit_kernel(const ulonglong2* __restrict__ raw, long long n,
+                                                         const K* __restrict__ A, const K* __restrict__ half,
+                                                         const unsigned long long* __restrict__ slot,
+                                                         const unsigned* __restrict__ count, unsigned mask,
+                                                         ulonglong2* __restrict__ keys_out,
+                                                         long long* __restrict__ counts_out,
+                                                         long long* __restrict__ n_unique, const Ctrl* ctrl) {
+    if (sort_whole<K>(ctrl, n)) return;
+    const long long m = ctrl->m;
+    const K* sorted = sorted_in(A, half, m);
+    for (long long j = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; j < m;
+         j += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const K k = sorted[j];
+        const unsigned long long h = key_hash(k);
+        unsigned s = static_cast<unsigned>(h >> 13) & mask;
+        for (unsigned it = 0; it < kProbeMax; ++it) {  // every listed key was placed within kProbeMax
+            const unsigned long long e = slot[s];
+            if (e == 0ULL || slot_holds(e, raw, k, h)) break;
+            s = (s + 1u) & mask;
+        }
+        keys_out[j] = k.wide();
+        counts_out[j] = count[s];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_unique = ctrl->bad != 0u ? -1 : m;
+}
+
+// KH: heads of runs per tile of the sorted stream.
+template <typename K>
+__device__ __forceinline__ bool run_head(const K* __restrict__ k, long long i) {
+    return i == 0 || !k[i].same(k[i - 1]);
+}
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) dedup_heads_kernel(const K* __restrict__ A, const K* __restrict__ B,
+                                                                   long long n, unsigned* __restrict__ heads_of,
+                                                                   const Ctrl* ctrl) {
+    if (!sort_whole<K>(ctrl, n)) return;
+    const K* k = sorted_in(A, B, n);
+    __shared__ unsigned total;
+    for (long long at = static_cast<long long>(blockIdx.x) * kTile; at < n;
+         at += static_cast<long long>(gridDim.x) * kTile) {
+        __syncthreads();
+        if (threadIdx.x == 0) total = 0u;
+        __syncthreads();
+        unsigned c = 0;
+        for (int t = threadIdx.x; t < kTile && at + t < n; t += kSortThreads) c += run_head(k, at + t) ? 1u : 0u;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&total, c);
+        __syncthreads();
+        if (threadIdx.x == 0) heads_of[at / kTile] = total;
     }
 }
 
@@ -154,7 +569,7 @@ __global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const unsigned* _
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* __restrict__ sums, long long m) {
+__device__ __forceinline__ void scan_top(unsigned* __restrict__ sums, long long m) {
     __shared__ unsigned sh[32];
     __shared__ unsigned carry;
     if (threadIdx.x == 0) carry = 0;
@@ -170,6 +585,15 @@ __global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* __restri
         __syncthreads();
     }
     if (threadIdx.x == 0) sums[m] = carry;
+}
+
+__global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* __restrict__ sums, long long m) {
+    scan_top(sums, m);
+}
+template <typename K>
+__global__ void __launch_bounds__(kScanBlock) dedup_scan_kernel(unsigned* __restrict__ sums, long long m, long long n,
+                                                                const Ctrl* ctrl) {
+    if (sort_whole<K>(ctrl, n)) scan_top(sums, m);
 }
 
 __global__ void __launch_bounds__(kScanBlock) scan_down_kernel(unsigned* __restrict__ a, long long n,
@@ -193,58 +617,126 @@ __global__ void __launch_bounds__(kScanBlock) scan_down_kernel(unsigned* __restr
 }
 
 
-// KU: head-of-run flags of the sorted keys (as 0/1 in `f`)
-__global__ void __launch_bounds__(256) dedup_flags_kernel(const ulonglong2* __restrict__ k, long long n,
-                                                          unsigned* __restrict__ f) {
-    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const ulonglong2 a = k[i];
-        bool head = i == 0;
-        if (!head) {
-            const ulonglong2 b = k[i - 1];
-            head = a.x != b.x || a.y != b.y;
-        }
-        f[i] = head ? 1u : 0u;
-    }
-}
 
-// KE: after the exclusive scan of the flags, each head writes its key and its position
-__global__ void __launch_bounds__(256) dedup_emit_kernel(const ulonglong2* __restrict__ k, long long n,
-                                                         const unsigned* __restrict__ pos,
-                                                         const unsigned* __restrict__ total_flags,
-                                                         ulonglong2* __restrict__ keys_out,
-                                                         long long* __restrict__ heads,
-                                                         long long* __restrict__ n_unique,
-                                                         const unsigned* __restrict__ flag) {
-    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const ulonglong2 a = k[i];
-        bool head = i == 0;
-        if (!head) {
-            const ulonglong2 b = k[i - 1];
-            head = a.x != b.x || a.y != b.y;
-        }
-        if (head) {
-            const unsigned j = pos[i];
-            keys_out[j] = a;
-            heads[j] = i;
+// KR: each head writes its key and its position at its rank.
+template <typename K>
+__global__ void __launch_bounds__(kSortThreads) dedup_runs_kernel(const K* __restrict__ A, const K* __restrict__ B,
+                                                                  long long n, const unsigned* __restrict__ before,
+                                                                  long long tiles, ulonglong2* __restrict__ keys_out,
+                                                                  long long* __restrict__ heads,
+                                                                  long long* __restrict__ n_unique, Ctrl* ctrl) {
+    if (!sort_whole<K>(ctrl, n)) return;
+    const K* k = sorted_in(A, B, n);
+    __shared__ unsigned warp_n[kSortThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (long long at = static_cast<long long>(blockIdx.x) * kTile; at < n;
+         at += static_cast<long long>(gridDim.x) * kTile) {
+        unsigned base = before[at / kTile];
+        for (int t0 = 0; t0 < kTile && at + t0 < n; t0 += kSortThreads) {
+            const long long i = at + t0 + threadIdx.x;
+            const bool head = i < n && run_head(k, i);
+            const unsigned m = __ballot_sync(0xffffffffu, head);
+            __syncthreads();
+            if (lane == 0) warp_n[warp] = __popc(m);
+            __syncthreads();
+            unsigned mine = base;
+            for (int w = 0; w < kSortThreads / 32; ++w) {
+                if (w < warp) mine += warp_n[w];
+                base += warp_n[w];
+            }
+            if (head) {
+                const unsigned j = mine + __popc(m & ((1u << lane) - 1u));
+                keys_out[j] = k[i].wide();
+                heads[j] = i;
+            }
         }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const long long u = static_cast<long long>(*total_flags);
+        const unsigned u = before[tiles];
         heads[u] = n;
-        *n_unique = (*flag != 0u) ? -1 : u;
+        ctrl->runs = u;
+        *n_unique = ctrl->bad != 0u ? -1 : static_cast<long long>(u);
     }
 }
 
 // KC: multiplicities = differences of consecutive head positions
 __global__ void __launch_bounds__(256) dedup_counts_kernel(const long long* __restrict__ heads,
-                                                           const unsigned* __restrict__ total_flags,
-                                                           long long* __restrict__ counts_out) {
-    const long long u = static_cast<long long>(*total_flags);
+                                                           long long* __restrict__ counts_out, const Ctrl* ctrl) {
+    const long long u = ctrl->runs;
     for (long long j = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; j < u;
          j += static_cast<long long>(gridDim.x) * blockDim.x)
         counts_out[j] = heads[j + 1] - heads[j];
+}
+
+__global__ void dedup_start_kernel(Ctrl* ctrl, unsigned full) {
+    *ctrl = Ctrl{0u, full, 0u, 0u};
+}
+
+template <typename K>
+cudaError_t dedup(const ulonglong2* raw, long long n, ulonglong2 high, ulonglong2* keys_out, long long* counts_out,
+                  long long* n_unique, unsigned char* W, const Layout& L, bool count, int sms, cudaStream_t s) {
+    K* A = reinterpret_cast<K*>(W + L.bufA);
+    K* B = reinterpret_cast<K*>(W + L.bufB);
+    long long* heads = reinterpret_cast<long long*>(W + L.heads);
+    // bufA's second half, on a 16-byte boundary (bufA's own rounding to 256 bytes covers the shift)
+    K* half = reinterpret_cast<K*>(W + L.bufA + (static_cast<size_t>(n) * 8 + 15) / 16 * 16);
+    unsigned long long* slot = reinterpret_cast<unsigned long long*>(W + L.bufB);
+    unsigned* counts = reinterpret_cast<unsigned*>(slot + L.slots);
+    unsigned* sums = reinterpret_cast<unsigned*>(W + L.sums);
+    Ctrl* ctrl = reinterpret_cast<Ctrl*>(W + L.ctrl);
+    const unsigned mask = L.slots - 1u;
+    const long long tiles = (n + kTile - 1) / kTile;
+    const unsigned grid = static_cast<unsigned>(std::min<long long>(tiles, 8LL * sms));
+    dedup_start_kernel<<<1, 1, 0, s>>>(ctrl, count ? 0u : 1u);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && count) {
+        constexpr size_t smem = CountTable<K>::bytes;
+        e = cudaMemsetAsync(slot, 0, static_cast<size_t>(L.slots) * 12, s);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(dedup_count_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(smem));
+        if (e == cudaSuccess) {
+            dedup_count_kernel<K><<<static_cast<unsigned>(sms), kCountThreads, smem, s>>>(raw, n, high, slot, counts,
+                                                                                         mask, ctrl);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) {
+            dedup_list_kernel<K><<<L.slots / (1024 * kListSlots), 1024, 0, s>>>(raw, slot, A, ctrl);
+            e = cudaGetLastError();
+        }
+    }
+    if (e == cudaSuccess) {
+        dedup_tile_kernel<K><<<grid, kSortThreads, 0, s>>>(raw, n, A, A, high, ctrl);
+        e = cudaGetLastError();
+    }
+    bool odd = false;
+    for (long long run = kTile; run < n && e == cudaSuccess; run *= 2) {
+        dedup_merge_kernel<K><<<grid, kSortThreads, 0, s>>>(A, B, half, odd, n, run, ctrl);
+        e = cudaGetLastError();
+        odd = !odd;
+    }
+    if (e == cudaSuccess && count) {
+        dedup_emit_kernel<K><<<4 * sms, 256, 0, s>>>(raw, n, A, half, slot, counts, mask, keys_out, counts_out,
+                                                    n_unique, ctrl);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        dedup_heads_kernel<K><<<grid, kSortThreads, 0, s>>>(A, B, n, sums, ctrl);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        dedup_scan_kernel<K><<<1, kScanBlock, 0, s>>>(sums, tiles, n, ctrl);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        dedup_runs_kernel<K><<<grid, kSortThreads, 0, s>>>(A, B, n, sums, tiles, keys_out, heads, n_unique, ctrl);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        dedup_counts_kernel<<<8 * sms, 256, 0, s>>>(heads, counts_out, ctrl);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 qc_status dfail(qc_status st, const char* msg) {
@@ -289,49 +781,27 @@ extern "C" qc_status qc_dedup(const uint64_t* raw, int64_t n_raw, int n_orb, uin
     const Layout L = layout(n);
     if (work_bytes < L.total) return dfail(QC_ERR_CAPACITY, "qc_dedup: workspace too small");
     unsigned char* W = static_cast<unsigned char*>(work);
-    ulonglong2* A = reinterpret_cast<ulonglong2*>(W + L.bufA);
-    ulonglong2* Bf = reinterpret_cast<ulonglong2*>(W + L.bufB);
-    long long* heads = reinterpret_cast<long long*>(W + L.heads);
-    unsigned* table = reinterpret_cast<unsigned*>(W + L.table);
-    unsigned* sums = reinterpret_cast<unsigned*>(W + L.sums);
-    unsigned* flag = reinterpret_cast<unsigned*>(W + L.flag);
-    const long long tiles = (n + kTile - 1) / kTile;
-    const unsigned blocks = static_cast<unsigned>((tiles + kWarpsPerBlock - 1) / kWarpsPerBlock);
     ulonglong2 high{};
     high.x = n_orb >= 64 ? 0ULL : ~((1ULL << n_orb) - 1ULL);
     high.y = n_orb >= 128 ? 0ULL : (n_orb <= 64 ? ~0ULL : ~((1ULL << (n_orb - 64)) - 1ULL));
-    cudaError_t e = cudaMemsetAsync(flag, 0, 16, s);
-    const int passes = (n_orb + 7) / 8;
-    const ulonglong2* src = reinterpret_cast<const ulonglong2*>(raw);
-    ulonglong2* dst = A;
-    for (int p = 0; p < passes && e == cudaSuccess; ++p) {
-        dedup_hist_kernel<<<blocks, 256, 0, s>>>(src, n, p, tiles, table, high, flag);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = qc::exclusive_scan_u32(table, static_cast<long long>(kBins) * tiles, sums, s);
-        if (e == cudaSuccess) {
-            dedup_scatter_kernel<<<blocks, 256, 0, s>>>(src, dst, n, p, tiles, table);
-            e = cudaGetLastError();
-        }
-        src = dst;
-        dst = (dst == A) ? Bf : A;
-    }
-    // src holds the sorted keys; the table area holds the flags and their scan
-    const unsigned gblocks = static_cast<unsigned>(std::min<long long>((n + 255) / 256, 8192));
-    if (e == cudaSuccess) {
-        dedup_flags_kernel<<<gblocks, 256, 0, s>>>(src, n, table);
-        e = cudaGetLastError();
-    }
-    const long long segs = (n + kScanSeg - 1) / kScanSeg;
-    if (e == cudaSuccess) e = qc::exclusive_scan_u32(table, n, sums, s);
-    if (e == cudaSuccess) {
-        dedup_emit_kernel<<<gblocks, 256, 0, s>>>(src, n, table, sums + segs, reinterpret_cast<ulonglong2*>(keys_out),
-                                                 heads, reinterpret_cast<long long*>(n_unique), flag);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-        dedup_counts_kernel<<<gblocks, 256, 0, s>>>(heads, sums + segs, reinterpret_cast<long long*>(counts_out));
-        e = cudaGetLastError();
-    }
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return dfail(QC_ERR_CUDA, cudaGetErrorString(e));
+    // counting reads the raw keys to the end, so outputs laid over them are written by the sort of
+    // the whole stream, which has read them all before it writes
+    auto over = [&](const void* p, size_t bytes) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(raw), b = reinterpret_cast<uintptr_t>(p);
+        return b < a + static_cast<size_t>(n) * 16 && a < b + bytes;
+    };
+    const size_t un = static_cast<size_t>(n);
+    const bool count = L.slots > 0 && !over(keys_out, un * 16) && !over(counts_out, un * 8) && !over(n_unique, 8);
+    const ulonglong2* r = reinterpret_cast<const ulonglong2*>(raw);
+    ulonglong2* ko = reinterpret_cast<ulonglong2*>(keys_out);
+    long long* co = reinterpret_cast<long long*>(counts_out);
+    long long* nu = reinterpret_cast<long long*>(n_unique);
+    e = n_orb <= 64 ? dedup<Key1>(r, n, high, ko, co, nu, W, L, count, sms, s)
+                    : dedup<Key2>(r, n, high, ko, co, nu, W, L, count, sms, s);
     if (e != cudaSuccess) return dfail(QC_ERR_CUDA, cudaGetErrorString(e));
     return QC_OK;
 }
