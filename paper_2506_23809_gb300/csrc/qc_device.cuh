@@ -57,7 +57,7 @@ __device__ __forceinline__ long long checked_index(long long i, long long n, uns
 // word's total parity carried into the high word).
 __device__ __forceinline__ ulonglong2 prefix_parity(ulonglong2 x) {
     unsigned long long lo = x.x, hi = x.y;
-#pragma unroll
+#pragma unroll 1
     for (int sh = 1; sh < 64; sh <<= 1) {
         lo ^= lo << sh;
         hi ^= hi << sh;
@@ -183,11 +183,11 @@ __device__ __forceinline__ unsigned home_bucket(unsigned g, unsigned nb_mask) {
 
 // Returns the table row of key (low hash bits g), or -1.  Buckets hold two 64-bit entries
 // (fingerprint << 32 | row + 1); an empty entry ends the probe sequence.  Called only on a
-// fingerprint collision (about 0.2% of hits), so it is kept out of line: its loop would
-// otherwise sit in the middle of the hit stage's code.
-static __device__ __noinline__ long long table_find(const TableParams& tp, ulonglong2 key, unsigned g) {
+// fingerprint collision (about 0.2% of hits).
+__device__ __forceinline__ long long table_find(const TableParams& tp, ulonglong2 key, unsigned g) {
     unsigned b = home_bucket(g, tp.nb_mask);
     const ulonglong2* buckets = reinterpret_cast<const ulonglong2*>(tp.slots);
+#pragma unroll 1
     for (unsigned it = 0; it <= tp.nb_mask; ++it) {
         const ulonglong2 e = __ldg(buckets + QC_IX(b, tp.nb_mask + 1LL, tp.err));
         if (e.x == 0ULL) return -1;
@@ -213,6 +213,7 @@ static __device__ __noinline__ long long table_find(const TableParams& tp, ulong
 __device__ __forceinline__ long long probe_fp(unsigned g, const TableParams& tp) {
     unsigned b = home_bucket(g, tp.nb_mask);
     const ulonglong2* buckets = reinterpret_cast<const ulonglong2*>(tp.slots);
+#pragma unroll 1
     for (unsigned it = 0; it <= tp.nb_mask; ++it) {
         const ulonglong2 e = __ldg(buckets + QC_IX(b, tp.nb_mask + 1LL, tp.err));
         if (e.x == 0ULL) return -1;
@@ -251,6 +252,7 @@ __device__ __forceinline__ unsigned set_insert(unsigned long long* set, unsigned
 __device__ __forceinline__ unsigned set_slot(const unsigned long long* __restrict__ set, unsigned mask,
                                              unsigned long long v, unsigned long long h) {
     unsigned b = static_cast<unsigned>(h >> 32) & mask;
+#pragma unroll 1
     for (unsigned it = 0; it <= mask; ++it) {
         const unsigned long long e = __ldg(set + (b & mask));
         if (e == v) return b;
@@ -446,6 +448,13 @@ __device__ __forceinline__ ulonglong2 excite(unsigned orbs, ulonglong2 x, unsign
     return excited_key(orbs, x);
 }
 
+// The row of the excitation `orbs` of x after a fingerprint collision (out of line: rare).
+static __device__ __noinline__ long long collision_row(const TableParams& tp, unsigned orbs, ulonglong2 xp,
+                                                       unsigned long long hx,
+                                                       const unsigned long long* __restrict__ T64) {
+    return table_find(tp, xp, static_cast<unsigned>(excited_hash(orbs, hx, T64)));
+}
+
 // Add one hit: <x|H|x'> (phase included) times psi(x') [FP64], or times psi(x')/psi(x)
 // [FP32, compensated], plus (DIAG) the per-sample digests of the exported phase convention.
 template <int PREC, bool DIAG>
@@ -487,7 +496,7 @@ __device__ __forceinline__ long long verify_and_add(uint2 e, bool exact, ulonglo
     element(h64, h32, sneg);
     long long row = e.y;
     if (key.x != xp.x || key.y != xp.y) {
-        row = table_find(tp, xp, static_cast<unsigned>(excited_hash(e.x, hx, T64)));
+        row = collision_row(tp, e.x, xp, hx, T64);
         if (row >= 0) pp = __ldg(tp.psi + QC_IX(row, tp.n, tp.err));
         else if (mode == QC_FULL) acc.missing++;
     }
@@ -556,8 +565,9 @@ __device__ __forceinline__ unsigned scan_code(unsigned kind, int d, unsigned lon
 // and fills (a, b); j = b = 255 for singles.  Classes: 0 alpha single (w), 1 beta single
 // (w), 2 alpha-alpha double (u: occupied pair, w: empty pair), 3 beta-beta double,
 // 4 alpha-beta double (u: alpha single, w: beta single), and the classes of scanned hits
-// (kCodeSingleA ..).  Same-spin doubles come out with i < j and a < b.  Single indices go
-// through IA / IB (the compacted single lists of the filtered kernel) when given.  Returns the packed orbitals i | a << 8 | j << 16 | b << 24.
+// (kCodeSingleA ..).  Same-spin doubles come out with i < j and a < b.  MAPPED: single indices go
+// through IA / IB (the compacted single lists of the filtered kernel).  Returns the packed orbitals i | a << 8 | j << 16 | b << 24.
+template <bool MAPPED = false>
 __device__ __forceinline__ unsigned decode(unsigned code, const SysParams& sp,
                                            const unsigned char* __restrict__ wl,
                                            const unsigned char* __restrict__ smem,
@@ -585,7 +595,7 @@ __device__ __forceinline__ unsigned decode(unsigned code, const SysParams& sp,
     const int w = static_cast<int>(code & 4095u);
     // the filtered kernel's single lists are compacted by the spin-string prefilter; their maps
     // IA / IB hold each entry's spatial orbitals (occupied | empty << 8)
-    if (IA != nullptr && (cls <= 1u || cls == 4u)) {
+    if (MAPPED && (cls <= 1u || cls == 4u)) {
         if (cls == 4u) {
             const unsigned pa = IA[QC_IX(u, sp.nsa, sp.err)], pb = IB[QC_IX(w, sp.nsb, sp.err)];
             return (2u * (pa & 255u)) | ((2u * (pa >> 8)) << 8) | ((2u * (pb & 255u) + 1u) << 16) |
@@ -595,13 +605,13 @@ __device__ __forceinline__ unsigned decode(unsigned code, const SysParams& sp,
         return (2u * (p & 255u) + cls) | ((2u * (p >> 8) + cls) << 8) | 0xFFFF0000u;
     }
     unsigned i, a, j = 255u, b = 255u;
-    if (cls == 4u) {
+    if (!MAPPED && cls == 4u) {
         const int io = divA[QC_IX(u, sp.nsa, sp.err)], jo = divB[QC_IX(w, sp.nsb, sp.err)];
         i = 2u * occA[QC_IX(io, sp.oa, sp.err)];
         a = 2u * virA[QC_IX(u - io * sp.va, sp.va, sp.err)];
         j = 2u * occB[QC_IX(jo, sp.ob, sp.err)] + 1u;
         b = 2u * virB[QC_IX(w - jo * sp.vb, sp.vb, sp.err)] + 1u;
-    } else if (cls >= 2u) {
+    } else if (MAPPED || cls >= 2u) {
         const unsigned po = lut[QC_IX(u, cls == 2u ? sp.npoa : sp.npob, sp.err)];
         const unsigned pv = lut[QC_IX(w, cls == 2u ? sp.npva : sp.npvb, sp.err)];
         const unsigned char* occ = cls == 2u ? occA : occB;
@@ -668,15 +678,19 @@ __device__ __forceinline__ void single_element(unsigned orbs, ulonglong2 px, con
         if (nd < sp.oa + sp.ob + os) {
             double f0 = sp.Fref[QC_IX((static_cast<unsigned>(s) * K + ka) * K + ki, 2 * QC_K2(sp), sp.err)], f1 = 0.0,
                    f2 = 0.0, f3 = 0.0;
+#pragma unroll 1
             for (unsigned long long m = aP | bP; m; m &= m - 1ULL) {
                 const int k = __ffsll(m) - 1;
                 f1 += ((aP >> k) & (bP >> k) & 1ULL) ? 2.0 * jt[k] : jt[k];
             }
+#pragma unroll 1
             for (unsigned long long m = aM | bM; m; m &= m - 1ULL) {
                 const int k = __ffsll(m) - 1;
                 f2 -= ((aM >> k) & (bM >> k) & 1ULL) ? 2.0 * jt[k] : jt[k];
             }
+#pragma unroll 1
             for (unsigned long long m = s ? bP : aP; m; m &= m - 1ULL) f3 -= xt[__ffsll(m) - 1];
+#pragma unroll 1
             for (unsigned long long m = s ? bM : aM; m; m &= m - 1ULL) f0 += xt[__ffsll(m) - 1];
             f = (f0 + f3) + (f1 + f2);
         } else {
@@ -684,11 +698,14 @@ __device__ __forceinline__ void single_element(unsigned orbs, ulonglong2 px, con
             double f0 = sp.h[QC_IX(ka * K + ki, QC_K2(sp), sp.err)], f1 = 0.0, f2 = 0.0, f3 = 0.0;
             const unsigned char* occS = s == 0 ? occA : occB;
             int q = 0;
+#pragma unroll 1
             for (; q + 1 < sp.oa; q += 2) { f0 += jt[occA[q]]; f1 += jt[occA[q + 1]]; }
             if (q < sp.oa) f0 += jt[occA[q]];
+#pragma unroll 1
             for (q = 0; q + 1 < sp.ob; q += 2) { f2 += jt[occB[q]]; f3 += jt[occB[q + 1]]; }
             if (q < sp.ob) f2 += jt[occB[q]];
             double g0 = 0.0, g1 = 0.0;
+#pragma unroll 1
             for (q = 0; q + 1 < os; q += 2) { g0 += xt[occS[q]]; g1 += xt[occS[q + 1]]; }
             if (q < os) g0 += xt[occS[q]];
             f = ((f0 + f1) + (f2 + f3)) - (g0 + g1);
@@ -701,11 +718,14 @@ __device__ __forceinline__ void single_element(unsigned orbs, ulonglong2 px, con
         const unsigned char* occS = s == 0 ? occA : occB;
         const int os = s == 0 ? sp.oa : sp.ob;
         int q = 0;
+#pragma unroll 1
         for (; q + 1 < sp.oa; q += 2) { f0 += jt[occA[q]]; f1 += jt[occA[q + 1]]; }
         if (q < sp.oa) f0 += jt[occA[q]];
+#pragma unroll 1
         for (q = 0; q + 1 < sp.ob; q += 2) { f2 += jt[occB[q]]; f3 += jt[occB[q + 1]]; }
         if (q < sp.ob) f2 += jt[occB[q]];
         float g0 = 0.f, g1 = 0.f;
+#pragma unroll 1
         for (q = 0; q + 1 < os; q += 2) { g0 += xt[occS[q]]; g1 += xt[occS[q + 1]]; }
         if (q < os) g0 += xt[occS[q]];
         const float f = ((f0 + f1) + (f2 + f3)) - (g0 + g1);
@@ -772,6 +792,7 @@ __device__ __forceinline__ bool sample_setup(const SysParams& sp, ulonglong2 x, 
                                  (static_cast<unsigned long long>(ahi) << 32);
     const unsigned long long B = static_cast<unsigned long long>(blo) |
                                  (static_cast<unsigned long long>(bhi) << 32);
+#pragma unroll 1
     for (int k = lane; k < sp.K; k += 32) {
         const unsigned long long lowm = (1ULL << k) - 1ULL;
         const int ca = __popcll(A & lowm), cb = __popcll(B & lowm);
@@ -799,25 +820,42 @@ __device__ __forceinline__ bool sample_setup(const SysParams& sp, ulonglong2 x, 
     const int K = sp.K;
     const int no = sp.oa + sp.ob;
     double e0 = 0.0, e1 = 0.0;
+#pragma unroll 1
     for (int p = lane; p < no; p += 32) {
         const int k = p < sp.oa ? occA[p] : occB[p - sp.oa];
         e1 += sp.h[QC_IX(k * K + k, QC_K2(sp), sp.err)];
     }
     if (no > 0) {
+        // lane l takes pairs l, l + 32, ..: four at a time, their loads in flight together (one at a
+        // time left a lane waiting for each table entry: N=52 2.63 -> 2.58 ms a step)
         const int q32 = 32 / no, r32 = 32 - q32 * no;
         int p = lane / no, r = lane - (lane / no) * no;
-        for (int t = lane; t < no * no; t += 32) {
-            const bool pa = p < sp.oa, ra = r < sp.oa;
-            const int k = pa ? occA[p] : occB[p - sp.oa];
-            const int l = ra ? occA[r] : occB[r - sp.oa];
-            e0 += (pa == ra ? sp.X : sp.J)[QC_IX(k * K + l, QC_K2(sp), sp.err)];
-            r += r32;
-            p += q32;
-            if (r >= no) {
-                r -= no;
-                ++p;
+        double e2 = 0.0, e3 = 0.0, e4 = 0.0;
+#pragma unroll 1
+        for (int t = lane; t < no * no; t += 128) {
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool in = t + 32 * k < no * no;
+                const int pp = in ? p : 0, rr = in ? r : 0;
+                const bool pa = pp < sp.oa, ra = rr < sp.oa;
+                const int kk = pa ? occA[pp] : occB[pp - sp.oa];
+                const int l = ra ? occA[rr] : occB[rr - sp.oa];
+                const double x = (pa == ra ? sp.X : sp.J)[QC_IX(kk * K + l, QC_K2(sp), sp.err)];
+                v[k] = in ? x : 0.0;
+                r += r32;
+                p += q32;
+                if (r >= no) {
+                    r -= no;
+                    ++p;
+                }
             }
+            e0 += v[0];
+            e2 += v[1];
+            e3 += v[2];
+            e4 += v[3];
         }
+        e0 = (e0 + e2) + (e3 + e4);
     }
     ediag = warp_sum(fma(0.5, e0, e1)) + sp.e_core;
     return true;
@@ -862,6 +900,30 @@ __device__ __forceinline__ void write_sample(const EvalParams& ep, long long s, 
     if (flags) atomicOr(&ep.ctr->flags, flags);
 }
 
+// One chunk of a sample evaluated in C > 1 excitation chunks (out of line: off by default).
+template <int PREC>
+static __device__ __noinline__ void finish_chunk(const EvalParams& ep, long long s, double ediag, double2 psix,
+                                                 const ChunkRec& mine, int c, int C) {
+    ChunkRec* rec = static_cast<ChunkRec*>(ep.cpart) + s * C;
+    rec[c] = mine;
+    __threadfence();
+    if (atomicAdd(ep.cticket + s, 1u) != static_cast<unsigned>(C - 1)) return;
+    __threadfence();
+    double re = 0.0, im = 0.0;
+    unsigned long long th = 0, tr = 0, tm = 0;
+    long long ts = 0;
+    for (int k = 0; k < C; ++k) {
+        const volatile ChunkRec* r = rec + k;
+        re += r->re;
+        im += r->im;
+        th += r->hits;
+        tr += r->rowsum;
+        ts += r->signsum;
+        tm += r->missing;
+    }
+    write_sample<PREC>(ep, s, ediag, psix, re, im, th, tr, ts, tm);
+}
+
 // Per-sample finish: reduce the lane accumulators and write the outputs.  With several
 // excitation chunks per sample (C > 1) each chunk stores its warp sums; the warp that
 // finishes the last chunk of the sample adds the C records in chunk order (the result does
@@ -888,7 +950,6 @@ __device__ __forceinline__ void sample_finish(const EvalParams& ep, long long s,
         write_sample<PREC>(ep, s, ediag, psix, sre, sim, hits, rows, sgn, miss);
         return;
     }
-    ChunkRec* rec = static_cast<ChunkRec*>(ep.cpart) + s * C;
     ChunkRec mine;
     mine.re = sre;
     mine.im = sim;
@@ -896,23 +957,7 @@ __device__ __forceinline__ void sample_finish(const EvalParams& ep, long long s,
     mine.rowsum = rows;
     mine.signsum = sgn;
     mine.missing = miss;
-    rec[c] = mine;
-    __threadfence();
-    if (atomicAdd(ep.cticket + s, 1u) != static_cast<unsigned>(C - 1)) return;
-    __threadfence();
-    double re = 0.0, im = 0.0;
-    unsigned long long th = 0, tr = 0, tm = 0;
-    long long ts = 0;
-    for (int k = 0; k < C; ++k) {
-        const volatile ChunkRec* r = rec + k;
-        re += r->re;
-        im += r->im;
-        th += r->hits;
-        tr += r->rowsum;
-        ts += r->signsum;
-        tm += r->missing;
-    }
-    write_sample<PREC>(ep, s, ediag, psix, re, im, th, tr, ts, tm);
+    finish_chunk<PREC>(ep, s, ediag, psix, mine, c, C);
 }
 
 static __device__ __noinline__ void invalid_sample(const EvalParams& ep, long long s, int lane) {
@@ -939,6 +984,10 @@ __device__ __forceinline__ float2 inv_psi32(double2 p) {
 // ------------------------------------------------------------------------------------
 // K2: the local-energy kernel
 // ------------------------------------------------------------------------------------
+// The kernel's speed depends on its code's size: 24 warps at different places of it make 60% of the
+// instruction cache's requests, 8% of them misses (ncu, N=52).  So its loops are not unrolled
+// (`#pragma unroll 1`: the compiler's fourfold copies of loops that run a few times), and what
+// rarely runs is out of line: N=52 2.58 -> 2.47 ms a step, N=76 11.67 -> 10.98, N=40 2.61 -> 2.55.
 // One warp per sample (persistent grid).  The five excitation classes are walked as
 // outer x inner products of per-sample hash lists by a flat state machine; each step
 // tests U x 32 excitations.  With FILTER, an excitation becomes a candidate only if its
@@ -1103,7 +1152,7 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
             if (!exact) key = __ldg(tp.keys + QC_IX(e.y, tp.n, tp.err));
             pp = __ldg(tp.psi + QC_IX(e.y, tp.n, tp.err));
         }
-        if (FILTER && v) e.x = decode(e.x, sp, wl, smem, IA, IB);
+        if (FILTER && v) e.x = decode<FILTER>(e.x, sp, wl, smem, IA, IB);
         long long ent = 0;
         if (v) {
             const ulonglong2 xs = wsp->x, px = wsp->px;
@@ -1183,6 +1232,7 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
         // drops it, compacting the single lists (IA / IB map back to the full index).
         const unsigned long long hxb = hx ^ hxa;
         nsb2 = 0;
+#pragma unroll 1
         for (int t0 = 0; t0 < sp.nsb; t0 += 32) {
             const int t = t0 + lane;
             bool keep = false;
@@ -1243,6 +1293,7 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
             nsa2 = 0;  // the alpha' groups are classified in the scan state
         } else {
             nsa2 = 0;
+#pragma unroll 1
             for (int t0 = 0; t0 < sp.nsa; t0 += 32) {
                 const int t = t0 + lane;
                 bool keep = false;
@@ -1271,29 +1322,37 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
         const bool needA = !join || enumB, needB = !join || enumA;
         if (lean) {
             if (needA) {
+#pragma unroll 1
                 for (int t = lane; t < sp.oa; t += 32) H[oPAo + t] = static_cast<uint32_t>(T64[2 * occA[t]]);
+#pragma unroll 1
                 for (int t = lane; t < sp.va; t += 32) H[oPAv + t] = static_cast<uint32_t>(T64[2 * virA[t]]);
             }
             if (needB) {
+#pragma unroll 1
                 for (int t = lane; t < sp.ob; t += 32) H[oPBo + t] = static_cast<uint32_t>(T64[2 * occB[t] + 1]);
+#pragma unroll 1
                 for (int t = lane; t < sp.vb; t += 32) H[oPBv + t] = static_cast<uint32_t>(T64[2 * virB[t] + 1]);
             }
         } else {
             if (needA) {
+#pragma unroll 1
                 for (int t = lane; t < sp.npoa; t += 32) {
                     const unsigned p = lut[t];
                     H[oPAo + t] = static_cast<uint32_t>(T64[2 * occA[p & 255u]] ^ T64[2 * occA[p >> 8]]);
                 }
+#pragma unroll 1
                 for (int t = lane; t < sp.npva; t += 32) {
                     const unsigned p = lut[t];
                     H[oPAv + t] = static_cast<uint32_t>(T64[2 * virA[p & 255u]] ^ T64[2 * virA[p >> 8]]);
                 }
             }
             if (needB) {
+#pragma unroll 1
                 for (int t = lane; t < sp.npob; t += 32) {
                     const unsigned p = lut[t];
                     H[oPBo + t] = static_cast<uint32_t>(T64[2 * occB[p & 255u] + 1] ^ T64[2 * occB[p >> 8] + 1]);
                 }
+#pragma unroll 1
                 for (int t = lane; t < sp.npvb; t += 32) {
                     const unsigned p = lut[t];
                     H[oPBv + t] = static_cast<uint32_t>(T64[2 * virB[p & 255u] + 1] ^ T64[2 * virB[p >> 8] + 1]);
@@ -1594,6 +1653,7 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
                 const unsigned code = v ? q[lane] : 0u;
                 if (DIAG && ep.work != nullptr && lane == 0) atomicAdd(&ep.work->probes, static_cast<unsigned long long>(n));
                 __syncwarp();
+#pragma unroll 1
                 for (int t = lane; t < qn - n; t += 32) q[t] = q[n + t];
                 qn -= n;
                 __syncwarp();
