@@ -1,14 +1,16 @@
 // qc_grad.cu -- Eq. 4 (Sec. II-A): the energy gradient
 //   d<E>/d theta_p = 2 Re < d_theta_p ln Psi*(n) (E_loc(n) - <E>) >_n
-// as a count-weighted average over the unique samples of one evaluation.  Two device steps:
+// as a count-weighted average over the unique samples of one evaluation.  Three device steps:
 //   K5 grad_weights_kernel   w_i = c_i (E_loc,i - Ebar) / W   (0 where E_loc is not finite)
 //   K6 grad_contract_kernel  partial_rp = sum over rows of chunk r of Re(w_i D_ip)
 //   K7 grad_finish_kernel    g_p = 2 sum_r partial_rp   (fixed order: deterministic)
 // Ebar and W come from the evaluation's device summary (written by the Eq. 1 reduction on
 // the same stream), so the call is asynchronous.  The contraction streams the n_u x P
 // complex rows D = d ln Psi* once from HBM (16 B per element, 16-byte streaming loads,
-// coalesced along a row) and spends two FP64 fused multiply-adds per element; at this GPU's
-// FP64 rate the arithmetic, not HBM, bounds it.
+// coalesced along a row): 0.97 ms for 1e5 x 4,096 at the 6.78 TB/s of a copy.  Two FP64
+// fused multiply-adds per element would take 1.38 ms (the FP64 pipe retires two per clock and
+// SM), so the real parts go through that pipe and the imaginary parts through integer
+// multiplications (FixedSum), which run beside it: 1.44 -> 1.01 ms a call, 6.5 TB/s.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,8 +22,9 @@
 
 namespace {
 
-constexpr int kGradThreads = 256;  // columns per CTA of the contraction
+constexpr int kGradThreads = 256;
 constexpr int kGradRowsMax = 256;  // rows of a chunk staged in shared memory at a time
+constexpr int kGradLoads = 4;      // row elements in flight per thread
 
 __device__ __forceinline__ double2 weight(const double2 e, const long long c, const qc_eloc_summary* sum) {
     const double W = sum->w;
@@ -39,61 +42,183 @@ __global__ void __launch_bounds__(256) grad_weights_kernel(const double2* __rest
         w[i] = weight(eloc[i], counts[i], sum);
 }
 
-// One CTA: kGradThreads consecutive columns of one chunk of rows.  The chunk's weights are
-// staged in shared memory; every thread then walks the rows of its column, four loads in
-// flight.
-__global__ void __launch_bounds__(kGradThreads) grad_contract_kernel(const double2* __restrict__ eloc,
-                                                                    const long long* __restrict__ counts,
-                                                                    long long n, const qc_eloc_summary* __restrict__ sum,
-                                                                    const double2* __restrict__ D, long long P,
-                                                                    long long rows_per_chunk, double* __restrict__ part) {
-    __shared__ double2 ws[kGradRowsMax];
-    const long long p = static_cast<long long>(blockIdx.x) * kGradThreads + threadIdx.x;
+// One staged row: its weight, and the imaginary weight's mantissa (the leading bit at bit 63),
+// biased exponent and the sign of -w.y as a mask.  A weight that is zero, subnormal or not
+// finite has an exponent that puts each of its products out of FixedSum's window.
+struct __align__(16) GradRow {
+    double2 w;
+    unsigned mhi, mlo;
+    int ex;
+    unsigned neg;
+};
+constexpr int kNoExponent = 1 << 20;
+
+__device__ __forceinline__ GradRow grad_row(double2 w) {
+    const unsigned hi = static_cast<unsigned>(__double2hiint(w.y)), lo = static_cast<unsigned>(__double2loint(w.y));
+    const int ex = static_cast<int>((hi >> 20) & 0x7ffu);
+    GradRow r;
+    r.w = w;
+    r.mhi = 0x80000000u | __funnelshift_l(lo, hi, 11);
+    r.mlo = lo << 11;
+    r.ex = ex == 0 ? -kNoExponent : ex == 0x7ff ? kNoExponent : ex;
+    r.neg = static_cast<unsigned>(~static_cast<int>(hi) >> 31);
+    return r;
+}
+
+// A sum of FP64 products in 96-bit fixed point, on the integer pipes.  A product is the top 64
+// bits of the mantissas' product (short of it by less than 3 units of its last place: 2^-60
+// relative), added without rounding at the place its exponent gives: the unit of the sum is
+// 2^(lim - kUnit), a product of exponents ex + ed sits `s` = lim - (ex + ed) places below the
+// top word, and at s >= kMinShift 2^8 of them cannot overflow.  What does not fit (s out of
+// [kMinShift, 64): a larger product than the sum was laid out for, one 2^-43 below it, a zero,
+// a subnormal, an infinity or NaN) goes to `slow`: the FP64 fused multiply-add.  A larger
+// product also moves the sum so far into the FP64 accumulator and lays it out anew, kMargin
+// places above that product.  So each product keeps at least the precision that the FP64 sum
+// gives it, over the whole range of FP64 (1e5 x 4,096: 2.4e-15 of the largest component off the
+// 64-bit sum, 2.5e-15 with FP64 throughout).
+constexpr int kMinShift = 9, kMargin = 12, kUnit = 2 * 1023 + 62 + 32;
+struct FixedSum {
+    unsigned a0 = 0, a1 = 0, a2 = 0;
+    int lim = -4 * kNoExponent;
+
+    // adds -w.y * d; returns false when the product does not fit (nothing is added then)
+    __device__ __forceinline__ bool add(const GradRow& r, double d) {
+        const unsigned hi = static_cast<unsigned>(__double2hiint(d)), lo = static_cast<unsigned>(__double2loint(d));
+        const int ed = static_cast<int>((hi >> 20) & 0x7ffu);
+        const int s = lim - r.ex - ed;
+        const bool ok = static_cast<unsigned>(ed - 1) < 0x7feu && static_cast<unsigned>(s - kMinShift) < 64u - kMinShift;
+        const unsigned keep = ok ? 0xffffffffu : 0u;
+        const unsigned mhi = 0x80000000u | __funnelshift_l(lo, hi, 11), mlo = lo << 11;
+        const unsigned neg = static_cast<unsigned>(static_cast<int>(hi) >> 31) ^ r.neg;
+        unsigned long long p = static_cast<unsigned long long>(mhi) * r.mhi + __umulhi(mhi, r.mlo);
+        p += __umulhi(mlo, r.mhi);
+        // one's complement for a negative product: a unit of the sum short, 2^-75 of the product
+        const unsigned m = neg & keep;
+        const unsigned pl = (static_cast<unsigned>(p) ^ neg) & keep, ph = (static_cast<unsigned>(p >> 32) ^ neg) & keep;
+        const unsigned f0 = __funnelshift_r(m, pl, s), f1 = __funnelshift_r(pl, ph, s);
+        const bool far = s >= 32;
+        // arithmetic shift of the signed product: the word above it is its sign
+        const unsigned f2 = __funnelshift_r(ph, m, s);
+        const unsigned w0 = far ? f1 : f0, w1 = far ? f2 : f1, w2 = far ? m : f2;
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(a0), "+r"(a1), "+r"(a2)
+            : "r"(w0), "r"(w1), "r"(w2));
+        return ok;
+    }
+    // the sum so far, which starts again from zero
+    __device__ __forceinline__ double take() {
+        const double low = __ull2double_rn((static_cast<unsigned long long>(a1) << 32) | a0);
+        const double v = fma(static_cast<double>(static_cast<int>(a2)), 18446744073709551616.0, low);
+        a0 = a1 = a2 = 0u;
+        return v == 0.0 ? 0.0 : ldexp(v, lim - kUnit);
+    }
+};
+
+struct GradSum {
+    FixedSum f;
+    double acc;
+};
+
+// A product that did not fit (by value, out of line: its operands stay in registers elsewhere).
+__device__ __noinline__ GradSum slow_product(GradSum g, double wy, int ex, double d) {
+    const int ed = (__double2hiint(d) >> 20) & 0x7ff;
+    g.acc = fma(-wy, d, g.acc);
+    if (ed > 0 && ed < 0x7ff && ex > 0 && ex < kNoExponent && g.f.lim - ex - ed < kMinShift) {
+        g.acc += g.f.take();
+        g.f.lim = ex + ed + kMinShift + kMargin;
+    }
+    return g;
+}
+
+// One CTA: 256 >> shift consecutive columns of one chunk of rows, the rows dealt over
+// 1 << shift groups of its threads, whose sums are added in a fixed order.  The chunk's
+// weights are staged in shared memory; every thread walks its rows of its column, kGradLoads
+// loads in flight.
+__global__ void __launch_bounds__(kGradThreads, 4)
+    grad_contract_kernel(const double2* __restrict__ eloc, const long long* __restrict__ counts,
+                         const double2* __restrict__ w, long long n, const qc_eloc_summary* __restrict__ sum,
+                         const double2* __restrict__ D, long long P, long long rows_per_chunk, int shift,
+                         double* __restrict__ part) {
+    __shared__ GradRow ws[kGradRowsMax];
+    const int cols = kGradThreads >> shift, groups = 1 << shift;
+    const int col = threadIdx.x & (cols - 1), grp = threadIdx.x / cols;
+    const long long p = static_cast<long long>(blockIdx.x) * cols + col;
     const long long r0 = static_cast<long long>(blockIdx.y) * rows_per_chunk;
     const long long r1 = r0 + rows_per_chunk < n ? r0 + rows_per_chunk : n;
-    double acc = 0.0;
+    GradSum g{};
     for (long long b = r0; b < r1; b += kGradRowsMax) {
         const int nb = static_cast<int>(r1 - b < kGradRowsMax ? r1 - b : kGradRowsMax);
         __syncthreads();
-        for (int t = threadIdx.x; t < nb; t += kGradThreads) ws[t] = weight(eloc[b + t], counts[b + t], sum);
+        for (int t = threadIdx.x; t < nb; t += kGradThreads)
+            ws[t] = grad_row(w != nullptr ? w[b + t] : weight(eloc[b + t], counts[b + t], sum));
         __syncthreads();
         if (p < P) {
-            const double2* row = D + b * P + p;
-            int t = 0;
-            for (; t + 4 <= nb; t += 4) {
-                const double2 d0 = __ldcs(row + (t + 0) * P);
-                const double2 d1 = __ldcs(row + (t + 1) * P);
-                const double2 d2 = __ldcs(row + (t + 2) * P);
-                const double2 d3 = __ldcs(row + (t + 3) * P);
-                // Re(w d) as two fused multiply-adds per element: the FP64 pipe, not HBM, is
-                // the narrower resource on this GPU, so no third FP64 operation per element
-                acc = fma(ws[t + 0].x, d0.x, acc);
-                acc = fma(-ws[t + 0].y, d0.y, acc);
-                acc = fma(ws[t + 1].x, d1.x, acc);
-                acc = fma(-ws[t + 1].y, d1.y, acc);
-                acc = fma(ws[t + 2].x, d2.x, acc);
-                acc = fma(-ws[t + 2].y, d2.y, acc);
-                acc = fma(ws[t + 3].x, d3.x, acc);
-                acc = fma(-ws[t + 3].y, d3.y, acc);
+            const double2* row = D + (b + grp) * P + p;
+            const long long step = static_cast<long long>(groups) * P;
+            int t = grp;
+            for (; t + (kGradLoads - 1) * groups < nb; t += kGradLoads * groups) {
+                double2 d[kGradLoads];
+#pragma unroll
+                for (int k = 0; k < kGradLoads; ++k) {
+                    d[k] = __ldcs(row);
+                    row += step;
+                }
+                bool ok[kGradLoads];
+#pragma unroll
+                for (int k = 0; k < kGradLoads; ++k) {
+                    const GradRow r = ws[t + k * groups];
+                    g.acc = fma(r.w.x, d[k].x, g.acc);
+                    ok[k] = g.f.add(r, d[k].y);
+                }
+                if (!(ok[0] && ok[1] && ok[2] && ok[3])) {
+#pragma unroll
+                    for (int k = 0; k < kGradLoads; ++k)
+                        if (!ok[k]) {
+                            const GradRow& r = ws[t + k * groups];
+                            g = slow_product(g, r.w.y, r.ex, d[k].y);
+                        }
+                }
             }
-            for (; t < nb; ++t) {
-                const double2 d = __ldcs(row + t * P);
-                acc = fma(ws[t].x, d.x, acc);
-                acc = fma(-ws[t].y, d.y, acc);
+            for (; t < nb; t += groups) {
+                const double2 d = __ldcs(row);
+                row += step;
+                const GradRow r = ws[t];
+                g.acc = fma(r.w.x, d.x, g.acc);
+                if (!g.f.add(r, d.y)) g = slow_product(g, r.w.y, r.ex, d.y);
             }
+            g.acc += g.f.take();
         }
     }
-    if (p < P) part[static_cast<long long>(blockIdx.y) * P + p] = acc;
+    if (groups > 1) {
+        __syncthreads();
+        double* sh = reinterpret_cast<double*>(ws);
+        sh[threadIdx.x] = g.acc;
+        __syncthreads();
+        if (grp != 0) return;
+        for (int k = 1; k < groups; ++k) g.acc += sh[k * cols + col];
+    }
+    if (p < P) part[static_cast<long long>(blockIdx.y) * P + p] = g.acc;
 }
 
-__global__ void __launch_bounds__(256) grad_finish_kernel(const double* __restrict__ part, int chunks, long long P,
-                                                          double* __restrict__ g) {
-    for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < P;
-         p += static_cast<long long>(gridDim.x) * blockDim.x) {
-        double s = 0.0;
-        for (int r = 0; r < chunks; ++r) s += part[static_cast<long long>(r) * P + p];
-        g[p] = 2.0 * s;
+// One CTA: 32 columns, each chunk's partials coalesced; 32 groups of threads take chunks
+// g, g + 32, .. and are added by halves (one thread a column walked all 512 chunks in 40 us).
+constexpr int kFinishGroups = 32;
+__global__ void __launch_bounds__(32 * kFinishGroups) grad_finish_kernel(const double* __restrict__ part, int chunks,
+                                                                        long long P, double* __restrict__ g) {
+    __shared__ double sh[kFinishGroups][32];
+    const int col = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const long long p = static_cast<long long>(blockIdx.x) * 32 + col;
+    double s = 0.0;
+    if (p < P)
+#pragma unroll 4
+        for (int r = grp; r < chunks; r += kFinishGroups) s += part[static_cast<long long>(r) * P + p];
+    sh[grp][col] = s;
+    __syncthreads();
+    for (int h = kFinishGroups / 2; h > 0; h >>= 1) {
+        if (grp < h) sh[grp][col] += sh[grp + h][col];
+        __syncthreads();
     }
+    if (grp == 0 && p < P) g[p] = 2.0 * sh[0][col];
 }
 
 // Row chunks of the contraction: a function of n only (not of the GPU), so the summation
@@ -102,6 +227,11 @@ int grad_chunks(long long n) {
     const long long c = (n + 63) / 64;
     return static_cast<int>(std::max<long long>(1, std::min<long long>(c, 512)));
 }
+
+// Row groups per CTA (as a shift): with 256 columns a CTA where that makes enough CTAs to fill
+// the GPU a few times over, else 32 columns and 8 rows at a time, so that few columns or few
+// rows still use the whole chip (a function of the sizes only, as the chunks).
+int grad_shift(long long P, int chunks) { return (P + kGradThreads - 1) / kGradThreads * chunks >= 1536 ? 0 : 3; }
 
 }  // namespace
 
@@ -147,16 +277,19 @@ extern "C" qc_status qc_eloc_grad(qc_eloc* H, const double* eloc, const int64_t*
                 if (e == cudaSuccess) H->gpart_cap = need;
             }
             if (e == cudaSuccess) {
-                const long long tiles = (n_par + kGradThreads - 1) / kGradThreads;
+                const int shift = grad_shift(n_par, chunks);
+                const long long cols = kGradThreads >> shift;
+                const long long tiles = (n_par + cols - 1) / cols;
                 if (tiles > 0x7fffffffLL) return fail(QC_ERR_CAPACITY, "n_par too large");
                 grad_contract_kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(chunks)), kGradThreads,
-                                       0, s>>>(e2, c, n_u, H->d_sum, reinterpret_cast<const double2*>(dconj), n_par,
-                                               rows, H->d_gpart);
+                                       0, s>>>(e2, c, reinterpret_cast<const double2*>(w_out), n_u, H->d_sum,
+                                               reinterpret_cast<const double2*>(dconj), n_par, rows, shift,
+                                               H->d_gpart);
                 e = cudaGetLastError();
             }
             if (e == cudaSuccess) {
-                const long long blocks = std::min<long long>((n_par + 255) / 256, 4096);
-                grad_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(H->d_gpart, chunks, n_par, g_out);
+                grad_finish_kernel<<<static_cast<unsigned>((n_par + 31) / 32), 32 * kFinishGroups, 0, s>>>(
+                    H->d_gpart, chunks, n_par, g_out);
                 e = cudaGetLastError();
             }
         }
