@@ -513,8 +513,10 @@ qc_status choose_config(qc_eloc* H, long long n_u, long long n_table, qc::Launch
     long long grid = H->opt_grid ? H->opt_grid : static_cast<long long>(per_sm) * H->sm_count;
     const long long cp = H->opt_chunk_pairs == 0 ? qc::kDefaultChunkPairs : H->opt_chunk_pairs;
     c.chunks = qc::exc_chunks(sp.pairs, cp);
-    const long long need = (n_u * c.chunks + c.warps - 1) / c.warps;
-    grid = std::max<long long>(1, std::min(grid, need));
+    // at most a CTA per work item: with fewer items than warps each CTA still gets some (packed
+    // into full CTAs, 1,000 samples ran on 42 of the 152 SMs)
+    grid = std::max<long long>(1, std::min(grid, n_u * c.chunks));
+    c.early = 1;
     c.grid = static_cast<int>(grid);
     return QC_OK;
 }
@@ -596,7 +598,9 @@ qc_status qc_eloc_eval(qc_eloc* H, const uint64_t* samples, const int64_t* count
         if (e != cudaSuccess) return cuda_fail(H, e, what); \
     } while (0)
     if (H->opt_timing) QC_CHK(cudaEventRecord(H->ev[0], s), "cudaEventRecord");
-    QC_CHK(cudaMemsetAsync(H->d_ctr, 0, sizeof(qc::Counters), s), "memset counters");
+    static_assert(sizeof(qc::Counters) % 16 == 0, "cleared in 16-byte stores");
+    qc::ClearList clear{};
+    clear.add(H->d_ctr, sizeof(qc::Counters));
 
     qc::TableParams tp{};
     tp.keys = tk;
@@ -616,10 +620,10 @@ qc_status qc_eloc_eval(qc_eloc* H, const uint64_t* samples, const int64_t* count
         tp.aset = aset;
         tp.bset = bset;
         tp.set_mask = tp.nb_mask;
-        QC_CHK(cudaMemsetAsync(H->d_sets, 0, 2 * nbuckets * sizeof(unsigned long long), s), "memset sets");
+        clear.add(H->d_sets, 2 * nbuckets * sizeof(unsigned long long));
     }
-    QC_CHK(cudaMemsetAsync(H->d_slots, 0, 2 * nbuckets * sizeof(unsigned long long), s), "memset table");
-    if (cfg.kernel == 2) QC_CHK(cudaMemsetAsync(H->d_filter, 0, (static_cast<size_t>(4) << fw), s), "memset filter");
+    clear.add(H->d_slots, 2 * nbuckets * sizeof(unsigned long long));
+    if (cfg.kernel == 2) clear.add(H->d_filter, static_cast<size_t>(4) << fw);
     // join index regions: slot keys, group sizes and starts, entries (strings, rows), sort space
     const bool join = cfg.join && nt > 0;
     auto a256 = [](size_t v) { return (v + 255) / 256 * 256; };
@@ -627,31 +631,32 @@ qc_status qc_eloc_eval(qc_eloc* H, const uint64_t* samples, const int64_t* count
     const size_t jo_len = JL.len, jo_start = JL.start, jo_ent = JL.ent, jo_ord = JL.ord, jo_ws = JL.ws;
     unsigned* jkey = nullptr;
     unsigned* jlen = nullptr;
+    unsigned* order = nullptr;
+    unsigned* pa = nullptr;
+    unsigned* pb = nullptr;
     const unsigned* join_order = nullptr;
     if (join) {
         st = qc::ensure_join(H, nt);
         if (st != QC_OK) return st;
         jkey = reinterpret_cast<unsigned*>(H->d_join);
         jlen = reinterpret_cast<unsigned*>(H->d_join + jo_len);
-        QC_CHK(cudaMemsetAsync(jlen, 0, 2 * nbuckets * sizeof(unsigned), s), "memset join sizes");
-    }
-    QC_CHK(qc::launch_build_table(tp, H->n_orb, H->na, H->nb, H->d_T, H->d_slots, H->d_filter, aset, bset,
-                                  H->d_ctr, s, jkey, jlen),
-           "build_table launch");
-    if (join) {
-        unsigned* jstart = reinterpret_cast<unsigned*>(H->d_join + jo_start);
-        ulonglong2* gent = reinterpret_cast<ulonglong2*>(H->d_join + jo_ent);
+        clear.add(jlen, (2 * nbuckets * sizeof(unsigned) + 15) / 16 * 16);
         // samples heavy first by the sizes of their own groups: the table's rows, or a caller's
         // samples no more numerous than its rows (the order's buffers hold one entry per row)
-        unsigned* order = nullptr;
-        unsigned* pa = nullptr;
-        unsigned* pb = nullptr;
         if (own_table || n_u <= nt) {
             order = reinterpret_cast<unsigned*>(H->d_join + jo_ord);
             pa = reinterpret_cast<unsigned*>(H->d_join + jo_ord + a256(static_cast<size_t>(nt) * 4));
             pb = reinterpret_cast<unsigned*>(H->d_join + jo_ord + 2 * a256(static_cast<size_t>(nt) * 4));
-            QC_CHK(cudaMemsetAsync(pa, 0, 2 * a256(static_cast<size_t>(nt) * 4), s), "memset sample order sizes");
+            clear.add(pa, 2 * a256(static_cast<size_t>(nt) * 4));
         }
+    }
+    QC_CHK(qc::launch_clear(clear, s), "clear launch");
+    QC_CHK(qc::launch_build_table(tp, H->n_orb, H->na, H->nb, H->d_T, H->d_slots, H->d_filter, aset, bset,
+                                  H->d_ctr, s, jkey, jlen, true),
+           "build_table launch");
+    if (join) {
+        unsigned* jstart = reinterpret_cast<unsigned*>(H->d_join + jo_start);
+        ulonglong2* gent = reinterpret_cast<ulonglong2*>(H->d_join + jo_ent);
         QC_CHK(qc::launch_join_index(tp, static_cast<unsigned>(nbuckets), H->d_join + jo_ws, jkey, jlen, jstart,
                                      gent, s, order, pa, pb,
                                      own_table ? nullptr : reinterpret_cast<const ulonglong2*>(samples), n_u, H->d_T),
@@ -712,7 +717,7 @@ qc_status qc_eloc_eval(qc_eloc* H, const uint64_t* samples, const int64_t* count
     }
     QC_CHK(qc::launch_eloc_main(H->sp, tp, ep, cfg, s), "main kernel launch");
     if (H->opt_timing) QC_CHK(cudaEventRecord(H->ev[2], s), "cudaEventRecord");
-    QC_CHK(qc::launch_reduce(ep, H->d_part, qc::reduce_blocks(n_u), H->d_sum, H->sp.pairs, s),
+    QC_CHK(qc::launch_reduce(ep, H->d_part, qc::reduce_blocks(n_u), H->d_sum, H->sp.pairs, s, true),
            "reduce launch");
     if (H->opt_timing) QC_CHK(cudaEventRecord(H->ev[3], s), "cudaEventRecord");
     if (out->summary)

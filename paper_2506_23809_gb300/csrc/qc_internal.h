@@ -214,6 +214,19 @@ struct LaunchCfg {
     int chunks;   // excitation chunks per sample
     int join;     // filtered kernel: sample-space join (short row groups scanned)
     int acap;     // join: slots of the per-warp alpha single list (0: all)
+    int early;    // launched while the stream's previous kernel still runs (launch_early)
+};
+
+// Byte ranges to zero in one launch: 16-byte aligned, sizes multiples of 16.
+struct ClearList {
+    static constexpr int kMax = 8;
+    void* p[kMax];
+    size_t bytes[kMax];
+    int n;
+    void add(void* q, size_t b) {
+        p[n] = q;
+        bytes[n++] = b;
+    }
 };
 
 // host-side launchers (qc_kernels.cu)
@@ -221,7 +234,8 @@ cudaError_t launch_build_table(const TableParams& tp, int n_orb, int na, int nb,
                                const unsigned long long* T, unsigned long long* slots,
                                uint32_t* filter, unsigned long long* aset,
                                unsigned long long* bset, Counters* ctr, cudaStream_t s,
-                               unsigned* jkey = nullptr, unsigned* jlen = nullptr);
+                               unsigned* jkey = nullptr, unsigned* jlen = nullptr, bool early = false);
+cudaError_t launch_clear(const ClearList& list, cudaStream_t s);
 cudaError_t launch_eloc_main(const SysParams& sp, const TableParams& tp, const EvalParams& ep,
                              const LaunchCfg& cfg, cudaStream_t s);
 // the same kernels with the hit lists and work counters compiled in (qc_kernels_diag.cu)
@@ -229,7 +243,7 @@ cudaError_t launch_eloc_main_diag(const SysParams& sp, const TableParams& tp, co
                                   const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t prepare_kernels_diag(size_t max_smem);
 cudaError_t launch_reduce(const EvalParams& ep, double* partials, int nblk,
-                          void* summary_dev, long long pairs_per_sample, cudaStream_t s);
+                          void* summary_dev, long long pairs_per_sample, cudaStream_t s, bool early = false);
 int max_active_ctas(int kernel, int precision, int unroll, int threads, size_t smem, int lean = 0, int join = 0,
                     int seg = 0);
 // batch: build every molecule's table in one launch (key_off: prefix of table sizes, device)

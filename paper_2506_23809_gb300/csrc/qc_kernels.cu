@@ -3,11 +3,14 @@
 // qc_main_kernel.cuh, its diagnostic instantiations in qc_kernels_diag.cu), K3 reduction.  The
 // device code they share with the batch kernels is in qc_device.cuh.
 #include <cstdint>
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "qc_main_kernel.cuh"
 
 namespace qc {
+
+namespace cg = cooperative_groups;
 
 int reduce_blocks(long long n) {
     // two rows per thread: enough blocks that every SM has a few (latency-bound loads)
@@ -33,32 +36,114 @@ __global__ void __launch_bounds__(256) build_table_kernel(TableParams tp, int n_
                                                           uint32_t* filter, unsigned long long* aset,
                                                           unsigned long long* bset, Counters* ctr,
                                                           unsigned* jkey, unsigned* jlen) {
+    let_next_start();
+    wait_previous();
     const long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r < tp.n) build_one(tp, n_orb, na, nb, T, slots, filter, aset, bset, ctr, r, jkey, jlen, 0u,
                             2u * (tp.set_mask + 1u));
 }
 
 __global__ void __launch_bounds__(kRedThreads) reduce_pass1(EvalParams ep, double* part) {
+    let_next_start();
+    wait_previous();
     reduce_pass1_body(ep, part, blockIdx.x, gridDim.x, 0, ep.n_u);
 }
 __global__ void __launch_bounds__(kRedThreads) reduce_pass2(EvalParams ep, double* part,
                                                             qc_eloc_summary* out, long long pairs_per_sample) {
+    wait_previous();
     reduce_pass2_body(ep, part, out, pairs_per_sample, blockIdx.x, gridDim.x, 0, ep.n_u);
+}
+
+// Both passes of a small sample set in one launch: a cluster of CTAs keeps its rows in registers
+// and exchanges its sums through distributed shared memory.  Up to kRedSmallRows rows; above, the
+// few SMs' FP64 rate (some ten operations a row at two per clock and SM) costs more than the
+// second launch.
+constexpr int kRedCluster = 8, kRedRowsPerThread = 4;
+constexpr long long kRedSmallRows = static_cast<long long>(kRedCluster) * kRedThreads * kRedRowsPerThread;
+
+__global__ void __cluster_dims__(kRedCluster, 1, 1) __launch_bounds__(kRedThreads)
+    reduce_small_kernel(EvalParams ep, qc_eloc_summary* out, long long pairs_per_sample) {
+    __shared__ RedSums sh[kRedWarps];
+    __shared__ double shd[kRedWarps];
+    __shared__ RedSums mine;
+    __shared__ double mine_var;
+    cg::cluster_group cl = cg::this_cluster();
+    wait_previous();
+    double2 e[kRedRowsPerThread];
+    long long c[kRedRowsPerThread];
+#pragma unroll
+    for (int k = 0; k < kRedRowsPerThread; ++k) {
+        const long long i = static_cast<long long>(k * kRedCluster + static_cast<int>(blockIdx.x)) * kRedThreads + threadIdx.x;
+        const bool in = i < ep.n_u;
+        e[k] = in ? ep.eloc[i] : make_double2(0.0, 0.0);
+        c[k] = in ? ep.counts[i] : 0;
+        if (!in) e[k].x = __longlong_as_double(0x7ff8000000000000LL);  // left out, like a NaN energy
+    }
+    RedSums v{};
+    bool neg = false;
+#pragma unroll
+    for (int k = 0; k < kRedRowsPerThread; ++k) red_row(e[k], c[k], v, neg);
+    if (neg) atomicOr(&ep.ctr->flags, QC_FLAG_NEG_COUNT);
+    v = block_sums(v, sh);
+    if (threadIdx.x == 0) {
+        mine = v;
+        __threadfence();  // the flags, for the CTA that writes the summary
+    }
+    cl.sync();
+    // every CTA adds the cluster's sums in the same order
+    RedSums t{};
+#pragma unroll
+    for (int r = 0; r < kRedCluster; ++r) red_add(t, *cl.map_shared_rank(&mine, r));
+    const double mr = t.re / static_cast<double>(t.w), mi = t.im / static_cast<double>(t.w);
+    double q = 0.0;
+#pragma unroll
+    for (int k = 0; k < kRedRowsPerThread; ++k) q += red_row_var(e[k], c[k], mr, mi);
+    q = block_sum(q, shd);
+    if (threadIdx.x == 0) mine_var = q;
+    cl.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double tv = 0.0;
+        for (int r = 0; r < kRedCluster; ++r) tv += *cl.map_shared_rank(&mine_var, r);
+        write_means(ep.ctr, t);
+        write_summary(ep.ctr, out, tv, ep.n_u, pairs_per_sample);
+    }
+    cl.sync();  // no CTA leaves while its sums are read
+}
+
+// Zeroes up to ClearList::kMax ranges (the tables and counters an evaluation starts from): one
+// launch in the place of four to six memsets.
+__global__ void __launch_bounds__(256) clear_kernel(const __grid_constant__ ClearList list) {
+    let_next_start();
+    const size_t step = static_cast<size_t>(gridDim.x) * blockDim.x;
+    for (int k = 0; k < list.n; ++k) {
+        uint4* p = static_cast<uint4*>(list.p[k]);
+        for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < list.bytes[k] / 16; i += step)
+            p[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 // ------------------------------------------------------------------------------------
 // host launchers
 // ------------------------------------------------------------------------------------
+cudaError_t launch_clear(const ClearList& list, cudaStream_t s) {
+    size_t most = 0;
+    for (int k = 0; k < list.n; ++k) most = list.bytes[k] > most ? list.bytes[k] : most;
+    // up to two 16-byte stores a thread and range, at most eight CTAs an SM
+    size_t blocks = (most / 16 + 511) / 512;
+    blocks = blocks < 1 ? 1 : blocks > 152 * 8 ? 152 * 8 : blocks;
+    clear_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(list);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_build_table(const TableParams& tp, int n_orb, int na, int nb,
                                const unsigned long long* T, unsigned long long* slots,
                                uint32_t* filter, unsigned long long* aset,
                                unsigned long long* bset, Counters* ctr, cudaStream_t s, unsigned* jkey,
-                               unsigned* jlen) {
+                               unsigned* jlen, bool early) {
     if (tp.n <= 0) return cudaSuccess;
     const long long blocks = (tp.n + 255) / 256;
-    build_table_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(tp, n_orb, na, nb, T, slots,
-                                                                      filter, aset, bset, ctr, jkey, jlen);
-    return cudaGetLastError();
+    return launch_early(build_table_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s, early, tp, n_orb, na,
+                        nb, T, slots, filter, aset, bset, ctr, jkey, jlen);
 }
 
 cudaError_t launch_eloc_main(const SysParams& sp, const TableParams& tp, const EvalParams& ep,
@@ -73,13 +158,15 @@ cudaError_t launch_eloc_main(const SysParams& sp, const TableParams& tp, const E
 }
 
 cudaError_t launch_reduce(const EvalParams& ep, double* partials, int nblk, void* summary_dev,
-                          long long pairs_per_sample, cudaStream_t s) {
-    reduce_pass1<<<nblk, kRedThreads, 0, s>>>(ep, partials);
-    cudaError_t e = cudaGetLastError();
+                          long long pairs_per_sample, cudaStream_t s, bool early) {
+    qc_eloc_summary* out = static_cast<qc_eloc_summary*>(summary_dev);
+    if (ep.n_u <= kRedSmallRows) {
+        return launch_early(reduce_small_kernel, dim3(kRedCluster), dim3(kRedThreads), 0, s, early, ep, out,
+                            pairs_per_sample);
+    }
+    const cudaError_t e = launch_early(reduce_pass1, dim3(nblk), dim3(kRedThreads), 0, s, early, ep, partials);
     if (e != cudaSuccess) return e;
-    reduce_pass2<<<nblk, kRedThreads, 0, s>>>(ep, partials,
-                                              static_cast<qc_eloc_summary*>(summary_dev), pairs_per_sample);
-    return cudaGetLastError();
+    return launch_early(reduce_pass2, dim3(nblk), dim3(kRedThreads), 0, s, early, ep, partials, out, pairs_per_sample);
 }
 
 int max_active_ctas(int kernel, int precision, int unroll, int threads, size_t smem, int lean, int join, int seg) {

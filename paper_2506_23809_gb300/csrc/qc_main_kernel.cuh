@@ -11,6 +11,24 @@
 
 namespace qc {
 
+// Launch with programmatic stream serialization (early) or plainly: the kernel may start while the
+// stream's previous kernel runs and synchronises with it by wait_previous.
+template <typename... P, typename... A>
+static cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool early,
+                                A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <int PREC, int U, bool FILTER, int LEAN, bool JOIN, bool DIAG, bool SEG = false>
 __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const __grid_constant__ SysParams sp,
                                                         const __grid_constant__ TableParams tp,
@@ -20,6 +38,9 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem + kOffBar);
     uint32_t* filt = reinterpret_cast<uint32_t*>(smem + kOffVar);
     const unsigned fbytes = FILTER ? (4u << tp.fw) : 0u;
+    let_next_start();
+    fill_cta_tables(sp, ep.T, smem);  // constants of the handle: before the previous kernel is waited for
+    wait_previous();
     if constexpr (FILTER) {
         if (threadIdx.x == 0) {
             mbar_init(bar, 1);
@@ -36,7 +57,6 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
             }
         }
     }
-    fill_cta_tables(sp, ep.T, smem);
     if constexpr (FILTER) {
         bool ready = false;
         const unsigned limit = ep.wait_limit > 0 ? static_cast<unsigned>(ep.wait_limit - 1) : kWaitLimit;
@@ -81,27 +101,23 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
 }
 
 template <int PREC, int LEAN, bool DIAG>
-static void launch_filtered(const SysParams& sp, const TableParams& tp, const EvalParams& ep, const LaunchCfg& c,
-                            cudaStream_t s) {
-    const dim3 grid(c.grid), block(32 * c.warps);
-    if (c.join && c.acap > 0) eloc_main_kernel<PREC, 4, true, LEAN, true, DIAG, true><<<grid, block, c.smem, s>>>(sp, tp, ep);
-    else if (c.join) eloc_main_kernel<PREC, 4, true, LEAN, true, DIAG><<<grid, block, c.smem, s>>>(sp, tp, ep);
-    else if (c.unroll == 1) eloc_main_kernel<PREC, 1, true, LEAN, false, DIAG><<<grid, block, c.smem, s>>>(sp, tp, ep);
-    else if (c.unroll == 2) eloc_main_kernel<PREC, 2, true, LEAN, false, DIAG><<<grid, block, c.smem, s>>>(sp, tp, ep);
-    else eloc_main_kernel<PREC, 4, true, LEAN, false, DIAG><<<grid, block, c.smem, s>>>(sp, tp, ep);
+static cudaError_t launch_filtered(const SysParams& sp, const TableParams& tp, const EvalParams& ep, const LaunchCfg& c,
+                                   cudaStream_t s) {
+    auto k = eloc_main_kernel<PREC, 4, true, LEAN, false, DIAG>;
+    if (c.join && c.acap > 0) k = eloc_main_kernel<PREC, 4, true, LEAN, true, DIAG, true>;
+    else if (c.join) k = eloc_main_kernel<PREC, 4, true, LEAN, true, DIAG>;
+    else if (c.unroll == 1) k = eloc_main_kernel<PREC, 1, true, LEAN, false, DIAG>;
+    else if (c.unroll == 2) k = eloc_main_kernel<PREC, 2, true, LEAN, false, DIAG>;
+    return launch_early(k, dim3(c.grid), dim3(32 * c.warps), c.smem, s, c.early != 0, sp, tp, ep);
 }
 
 template <int PREC, bool DIAG>
 static cudaError_t launch_main_p(const SysParams& sp, const TableParams& tp, const EvalParams& ep,
                                  const LaunchCfg& c, cudaStream_t s) {
-    if (c.kernel != 2) {
-        eloc_main_kernel<PREC, 1, false, 0, false, DIAG><<<dim3(c.grid), dim3(32 * c.warps), c.smem, s>>>(sp, tp, ep);
-    } else if (c.lean) {
-        launch_filtered<PREC, 1, DIAG>(sp, tp, ep, c, s);
-    } else {
-        launch_filtered<PREC, 0, DIAG>(sp, tp, ep, c, s);
-    }
-    return cudaGetLastError();
+    if (c.kernel != 2)
+        return launch_early(eloc_main_kernel<PREC, 1, false, 0, false, DIAG>, dim3(c.grid), dim3(32 * c.warps), c.smem, s,
+                            c.early != 0, sp, tp, ep);
+    return c.lean ? launch_filtered<PREC, 1, DIAG>(sp, tp, ep, c, s) : launch_filtered<PREC, 0, DIAG>(sp, tp, ep, c, s);
 }
 
 // the join is built with U = 4 only; seg: its alpha list is capped (enumerated in segments)
