@@ -221,17 +221,29 @@ __global__ void __launch_bounds__(32 * kFinishGroups) grad_finish_kernel(const d
     if (grp == 0 && p < P) g[p] = 2.0 * sh[0][col];
 }
 
-// Row chunks of the contraction: a function of n only (not of the GPU), so the summation
-// order, and the result, are the same everywhere.
-int grad_chunks(long long n) {
-    const long long c = (n + 63) / 64;
-    return static_cast<int>(std::max<long long>(1, std::min<long long>(c, 512)));
+// The contraction's split: columns per CTA (256 >> shift), rows per chunk and chunks.  A function
+// of the sizes only (not of the GPU), so the summation order, and the result, are the same
+// everywhere.  Up to 128 columns the CTA's threads share the rows; the chunks fill whole waves of
+// kGradWave CTAs (four on each of 152 SMs) with at most 256 rows a CTA and at least 8 a thread,
+// as a CTA starts and ends with some twenty FP64 operations a thread (5,723 x 2,816: 64-row
+// chunks of 256 columns 80 us, of 32 columns 126 us).
+constexpr long long kGradWave = 608, kGradChunksMax = 512;
+struct GradSplit {
+    int shift, chunks;
+    long long tiles, rows;
+};
+GradSplit grad_split(long long n, long long P) {
+    GradSplit g{};
+    while (g.shift < 3 && P <= (kGradThreads >> (g.shift + 1))) ++g.shift;
+    const long long cols = kGradThreads >> g.shift;
+    g.tiles = (P + cols - 1) / cols;
+    const long long waves = std::max<long long>(1, (g.tiles * ((n + 255) / 256) + kGradWave - 1) / kGradWave);
+    const long long most = std::min<long long>(kGradChunksMax, (n + (8LL << g.shift) - 1) / (8LL << g.shift));
+    const long long chunks = std::max<long long>(1, std::min(most, kGradWave * waves / g.tiles));
+    g.rows = (n + chunks - 1) / chunks;
+    g.chunks = static_cast<int>((n + g.rows - 1) / g.rows);
+    return g;
 }
-
-// Row groups per CTA (as a shift): with 256 columns a CTA where that makes enough CTAs to fill
-// the GPU a few times over, else 32 columns and 8 rows at a time, so that few columns or few
-// rows still use the whole chip (a function of the sizes only, as the chunks).
-int grad_shift(long long P, int chunks) { return (P + kGradThreads - 1) / kGradThreads * chunks >= 1536 ? 0 : 3; }
 
 }  // namespace
 
@@ -266,8 +278,8 @@ extern "C" qc_status qc_eloc_grad(qc_eloc* H, const double* eloc, const int64_t*
         if (n_u == 0) {
             e = cudaMemsetAsync(g_out, 0, static_cast<size_t>(n_par) * sizeof(double), s);
         } else {
-            const int chunks = grad_chunks(n_u);
-            const long long rows = (n_u + chunks - 1) / chunks;
+            const GradSplit sp = grad_split(n_u, n_par);
+            const int chunks = sp.chunks;
             const size_t need = static_cast<size_t>(chunks) * static_cast<size_t>(n_par);
             if (need > H->gpart_cap) {
                 if (H->d_gpart) cudaFree(H->d_gpart);
@@ -277,13 +289,10 @@ extern "C" qc_status qc_eloc_grad(qc_eloc* H, const double* eloc, const int64_t*
                 if (e == cudaSuccess) H->gpart_cap = need;
             }
             if (e == cudaSuccess) {
-                const int shift = grad_shift(n_par, chunks);
-                const long long cols = kGradThreads >> shift;
-                const long long tiles = (n_par + cols - 1) / cols;
-                if (tiles > 0x7fffffffLL) return fail(QC_ERR_CAPACITY, "n_par too large");
-                grad_contract_kernel<<<dim3(static_cast<unsigned>(tiles), static_cast<unsigned>(chunks)), kGradThreads,
+                if (sp.tiles > 0x7fffffffLL) return fail(QC_ERR_CAPACITY, "n_par too large");
+                grad_contract_kernel<<<dim3(static_cast<unsigned>(sp.tiles), static_cast<unsigned>(chunks)), kGradThreads,
                                        0, s>>>(e2, c, reinterpret_cast<const double2*>(w_out), n_u, H->d_sum,
-                                               reinterpret_cast<const double2*>(dconj), n_par, rows, shift,
+                                               reinterpret_cast<const double2*>(dconj), n_par, sp.rows, sp.shift,
                                                H->d_gpart);
                 e = cudaGetLastError();
             }

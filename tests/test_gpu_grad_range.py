@@ -53,8 +53,8 @@ def _exact(w, d):
 
 
 # rows: one, a partial load group, the edges of a 64-row chunk, and of a 256-row stage in use
-# (above 131,072 rows a chunk has more than 256); columns: the edges of a 32-column tile, and
-# the two sides of the 256-column rule (1,536 CTAs)
+# (above 131,072 rows of few columns a chunk has more than 256); columns: the edges of the 32- to
+# 256-column tiles
 @pytest.mark.parametrize("n_u,P", [(1, 1), (3, 33), (63, 32), (65, 31), (257, 300), (4000, 6145), (131_073, 65),
                                    (33_000, 640), (33_000, 768)])
 def test_grad_edges(B, n_u, P):
