@@ -1775,21 +1775,22 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return v;
 }
 
-// One row of pass 1 and of pass 2.
+// One row of pass 1 and of pass 2 (every rounding written out: all forms of the reduction give the
+// same bits).
 __device__ __forceinline__ void red_row(double2 e, long long c, RedSums& v, bool& neg) {
     if (c < 0) {
         neg = true;
     } else if (isfinite(e.x) && isfinite(e.y)) {
         v.w += c;
-        v.re += static_cast<double>(c) * e.x;
-        v.im += static_cast<double>(c) * e.y;
+        v.re = __fma_rn(static_cast<double>(c), e.x, v.re);
+        v.im = __fma_rn(static_cast<double>(c), e.y, v.im);
         v.used++;
     }
 }
-__device__ __forceinline__ double red_row_var(double2 e, long long c, double mr, double mi) {
-    if (c < 0 || !isfinite(e.x) || !isfinite(e.y)) return 0.0;
+__device__ __forceinline__ double red_row_var(double2 e, long long c, double mr, double mi, double v) {
+    if (c < 0 || !isfinite(e.x) || !isfinite(e.y)) return v;
     const double dr = e.x - mr, di = e.y - mi;
-    return static_cast<double>(c) * (dr * dr + di * di);
+    return __fma_rn(static_cast<double>(c), __fma_rn(dr, dr, __dmul_rn(di, di)), v);
 }
 
 __device__ __forceinline__ void write_means(Counters* c, const RedSums& t) {
@@ -1881,7 +1882,7 @@ __device__ __forceinline__ void reduce_pass2_body(const EvalParams& ep, double* 
     double v = 0.0;
     for (long long i = lo + static_cast<long long>(bid) * kRedThreads + threadIdx.x; i < hi;
          i += static_cast<long long>(nblk) * kRedThreads)
-        v += red_row_var(ep.eloc[i], ep.counts[i], mr, mi);
+        v = red_row_var(ep.eloc[i], ep.counts[i], mr, mi, v);
     v = block_sum(v, shd);
     if (threadIdx.x == 0) {
         part[4 * bid] = v;

@@ -55,57 +55,77 @@ __global__ void __launch_bounds__(kRedThreads) reduce_pass2(EvalParams ep, doubl
 }
 
 // Both passes of a small sample set in one launch: a cluster of CTAs keeps its rows in registers
-// and exchanges its sums through distributed shared memory.  Up to kRedSmallRows rows; above, the
-// few SMs' FP64 rate (some ten operations a row at two per clock and SM) costs more than the
-// second launch.
-constexpr int kRedCluster = 8, kRedRowsPerThread = 4;
-constexpr long long kRedSmallRows = static_cast<long long>(kRedCluster) * kRedThreads * kRedRowsPerThread;
+// and exchanges its sums through distributed shared memory.  Each CTA stands for two blocks of the
+// grid-wide passes and every sum is added in their order, so the summary has the same bits
+// as theirs (a batch reduces its molecules by the passes).  Up to kRedSmallRows rows, two a thread;
+// above, the few SMs' FP64 rate (some ten operations a row at two per clock and SM) costs more
+// than the second launch.
+constexpr int kRedCluster = 8, kRedVirtual = 2;
+constexpr long long kRedSmallRows = static_cast<long long>(kRedCluster) * kRedVirtual * kRedThreads * 2;
 
 __global__ void __cluster_dims__(kRedCluster, 1, 1) __launch_bounds__(kRedThreads)
-    reduce_small_kernel(EvalParams ep, qc_eloc_summary* out, long long pairs_per_sample) {
+    reduce_small_kernel(EvalParams ep, qc_eloc_summary* out, long long pairs_per_sample, int nblk) {
     __shared__ RedSums sh[kRedWarps];
     __shared__ double shd[kRedWarps];
-    __shared__ RedSums mine;
-    __shared__ double mine_var;
+    __shared__ RedSums mine[kRedVirtual], total;
+    __shared__ double mine_var[kRedVirtual];
     cg::cluster_group cl = cg::this_cluster();
     wait_previous();
-    double2 e[kRedRowsPerThread];
-    long long c[kRedRowsPerThread];
+    const int lane = threadIdx.x & 31;
+    double2 e[kRedVirtual][2];
+    long long c[kRedVirtual][2];
 #pragma unroll
-    for (int k = 0; k < kRedRowsPerThread; ++k) {
-        const long long i = static_cast<long long>(k * kRedCluster + static_cast<int>(blockIdx.x)) * kRedThreads + threadIdx.x;
-        const bool in = i < ep.n_u;
-        e[k] = in ? ep.eloc[i] : make_double2(0.0, 0.0);
-        c[k] = in ? ep.counts[i] : 0;
-        if (!in) e[k].x = __longlong_as_double(0x7ff8000000000000LL);  // left out, like a NaN energy
-    }
-    RedSums v{};
+    for (int b = 0; b < kRedVirtual; ++b)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int vb = b * kRedCluster + static_cast<int>(blockIdx.x);
+            const long long i = static_cast<long long>(vb + k * nblk) * kRedThreads + threadIdx.x;
+            const bool in = vb < nblk && i < ep.n_u;
+            // a row past the end is left out like one of a NaN energy
+            e[b][k] = in ? ep.eloc[i] : make_double2(__longlong_as_double(0x7ff8000000000000LL), 0.0);
+            c[b][k] = in ? ep.counts[i] : 0;
+        }
     bool neg = false;
 #pragma unroll
-    for (int k = 0; k < kRedRowsPerThread; ++k) red_row(e[k], c[k], v, neg);
-    if (neg) atomicOr(&ep.ctr->flags, QC_FLAG_NEG_COUNT);
-    v = block_sums(v, sh);
-    if (threadIdx.x == 0) {
-        mine = v;
-        __threadfence();  // the flags, for the CTA that writes the summary
+    for (int b = 0; b < kRedVirtual; ++b) {
+        RedSums v{};
+        red_row(e[b][0], c[b][0], v, neg);
+        red_row(e[b][1], c[b][1], v, neg);
+        v = block_sums(v, sh);
+        if (threadIdx.x == 0) mine[b] = v;
+    }
+    if (neg) {
+        atomicOr(&ep.ctr->flags, QC_FLAG_NEG_COUNT);
+        __threadfence();  // for the CTA that writes the summary
     }
     cl.sync();
-    // every CTA adds the cluster's sums in the same order
-    RedSums t{};
+    if (threadIdx.x < 32) {
+        RedSums t{};
+        if (lane < nblk) t = cl.map_shared_rank(mine, lane % kRedCluster)[lane / kRedCluster];
 #pragma unroll
-    for (int r = 0; r < kRedCluster; ++r) red_add(t, *cl.map_shared_rank(&mine, r));
-    const double mr = t.re / static_cast<double>(t.w), mi = t.im / static_cast<double>(t.w);
-    double q = 0.0;
+        for (int o = 16; o > 0; o >>= 1)
+            red_add(t, RedSums{__shfl_down_sync(QC_FULLMASK, t.re, o), __shfl_down_sync(QC_FULLMASK, t.im, o),
+                               __shfl_down_sync(QC_FULLMASK, t.w, o), __shfl_down_sync(QC_FULLMASK, t.used, o)});
+        red_add(t, RedSums{});
+        if (lane == 0) total = t;
+    }
+    __syncthreads();
+    const double mr = total.re / static_cast<double>(total.w), mi = total.im / static_cast<double>(total.w);
 #pragma unroll
-    for (int k = 0; k < kRedRowsPerThread; ++k) q += red_row_var(e[k], c[k], mr, mi);
-    q = block_sum(q, shd);
-    if (threadIdx.x == 0) mine_var = q;
+    for (int b = 0; b < kRedVirtual; ++b) {
+        double q = red_row_var(e[b][0], c[b][0], mr, mi, 0.0);
+        q = block_sum(red_row_var(e[b][1], c[b][1], mr, mi, q), shd);
+        if (threadIdx.x == 0) mine_var[b] = q;
+    }
     cl.sync();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double tv = 0.0;
-        for (int r = 0; r < kRedCluster; ++r) tv += *cl.map_shared_rank(&mine_var, r);
-        write_means(ep.ctr, t);
-        write_summary(ep.ctr, out, tv, ep.n_u, pairs_per_sample);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        double tv = lane < nblk ? cl.map_shared_rank(mine_var, lane % kRedCluster)[lane / kRedCluster] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tv += __shfl_down_sync(QC_FULLMASK, tv, o);
+        if (lane == 0) {
+            write_means(ep.ctr, total);
+            write_summary(ep.ctr, out, tv, ep.n_u, pairs_per_sample);
+        }
     }
     cl.sync();  // no CTA leaves while its sums are read
 }
@@ -162,7 +182,7 @@ cudaError_t launch_reduce(const EvalParams& ep, double* partials, int nblk, void
     qc_eloc_summary* out = static_cast<qc_eloc_summary*>(summary_dev);
     if (ep.n_u <= kRedSmallRows) {
         return launch_early(reduce_small_kernel, dim3(kRedCluster), dim3(kRedThreads), 0, s, early, ep, out,
-                            pairs_per_sample);
+                            pairs_per_sample, nblk);
     }
     const cudaError_t e = launch_early(reduce_pass1, dim3(nblk), dim3(kRedThreads), 0, s, early, ep, partials);
     if (e != cudaSuccess) return e;
