@@ -559,6 +559,8 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* s
 __global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const unsigned* __restrict__ a, long long n,
                                                                unsigned* __restrict__ sums) {
     __shared__ unsigned sh[32];
+    qc::let_next_start();
+    qc::wait_previous();
     const long long base = static_cast<long long>(blockIdx.x) * kScanSeg + threadIdx.x * kScanItems;
     unsigned v = 0;
 #pragma unroll
@@ -588,6 +590,8 @@ __device__ __forceinline__ void scan_top(unsigned* __restrict__ sums, long long 
 }
 
 __global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* __restrict__ sums, long long m) {
+    qc::let_next_start();
+    qc::wait_previous();
     scan_top(sums, m);
 }
 template <typename K>
@@ -596,9 +600,11 @@ __global__ void __launch_bounds__(kScanBlock) dedup_scan_kernel(unsigned* __rest
     if (sort_whole<K>(ctrl, n)) scan_top(sums, m);
 }
 
-__global__ void __launch_bounds__(kScanBlock) scan_down_kernel(unsigned* __restrict__ a, long long n,
+__global__ void __launch_bounds__(kScanBlock) scan_down_kernel(const unsigned* a, unsigned* out, long long n,
                                                                const unsigned* __restrict__ sums) {
     __shared__ unsigned sh[32];
+    qc::let_next_start();
+    qc::wait_previous();
     const long long base = static_cast<long long>(blockIdx.x) * kScanSeg + threadIdx.x * kScanItems;
     unsigned v[kScanItems], s = 0;
 #pragma unroll
@@ -611,7 +617,7 @@ __global__ void __launch_bounds__(kScanBlock) scan_down_kernel(unsigned* __restr
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k)
         if (base + k < n) {
-            a[base + k] = run;
+            out[base + k] = run;
             run += v[k];
         }
 }
@@ -746,15 +752,16 @@ qc_status dfail(qc_status st, const char* msg) {
 
 }  // namespace
 
-// Exclusive prefix sum of a u32 array in place (segment sums, a scan of the sums, segment
-// scans); also the join index's group starts (qc_join.cu).
-cudaError_t qc::exclusive_scan_u32(unsigned* a, long long n, unsigned* sums, cudaStream_t s) {
+// Exclusive prefix sum of a u32 array, in place or into another (segment sums, a scan of the
+// sums, segment scans): the join index's group starts and digit offsets (qc_join.cu).
+cudaError_t qc::exclusive_scan_u32(const unsigned* in, unsigned* out, long long n, unsigned* sums, cudaStream_t s) {
     const long long segs = (n + kScanSeg - 1) / kScanSeg;
     if (segs == 0) return cudaSuccess;
-    scan_sums_kernel<<<static_cast<unsigned>(segs), kScanBlock, 0, s>>>(a, n, sums);
-    scan_top_kernel<<<1, kScanBlock, 0, s>>>(sums, segs);
-    scan_down_kernel<<<static_cast<unsigned>(segs), kScanBlock, 0, s>>>(a, n, sums);
-    return cudaGetLastError();
+    const dim3 grid(static_cast<unsigned>(segs)), block(kScanBlock);
+    cudaError_t e = launch_early(scan_sums_kernel, grid, block, 0, s, true, in, n, sums);
+    if (e == cudaSuccess) e = launch_early(scan_top_kernel, dim3(1), block, 0, s, true, sums, segs);
+    if (e == cudaSuccess) e = launch_early(scan_down_kernel, grid, block, 0, s, true, in, out, n, sums);
+    return e;
 }
 
 extern "C" int64_t qc_dedup_workspace_bytes(int64_t n_raw) {

@@ -267,14 +267,6 @@ __device__ __forceinline__ bool set_contains(const unsigned long long* __restric
     return set_slot(set, mask, v, h) != kNoSlot;
 }
 
-// Programmatic dependent launch.  wait_previous: the stream's previous kernel has completed and its
-// writes are visible (returns at once in a kernel launched without launch_early); every kernel so
-// launched calls it in every thread before it reads or writes device memory that another kernel
-// touches, so completion stays transitive along the stream.  let_next_start: the stream's next
-// kernel, if launched by launch_early, may become resident from here on.
-__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Insert row r of the table: validation, filter bits, spin-string sets, bucket entry.  With
 // jkey (the sample-space join index), also the row's two set slots as sort keys -- jkey[r]
 // jbase + the alpha slot, jkey[n + r] jbase + set size + the beta slot (jsent for a row that

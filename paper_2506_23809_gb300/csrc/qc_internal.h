@@ -217,6 +217,32 @@ struct LaunchCfg {
     int early;    // launched while the stream's previous kernel still runs (launch_early)
 };
 
+// Programmatic dependent launch.  wait_previous: the stream's previous kernel has completed and its
+// writes are visible (returns at once in a kernel launched without launch_early); every kernel so
+// launched calls it in every thread before it reads or writes device memory that another kernel
+// touches, so completion stays transitive along the stream.  let_next_start: the stream's next
+// kernel, if launched by launch_early, may become resident from here on.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launch with programmatic stream serialization (early) or plainly: the kernel may start while the
+// stream's previous kernel runs and synchronises with it by wait_previous.
+template <typename... P, typename... A>
+static cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool early,
+                                A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Byte ranges to zero in one launch: 16-byte aligned, sizes multiples of 16.
 struct ClearList {
     static constexpr int kMax = 8;
@@ -285,7 +311,7 @@ cudaError_t launch_join_batch(const MolParams* mols, const unsigned* slot_base, 
                               const unsigned* row_base = nullptr, unsigned* order = nullptr,
                               unsigned* pa = nullptr, unsigned* pb = nullptr);
 // in-place exclusive prefix sum of n u32 (qc_dedup.cu); sums: (n / 4096 + 2) u32 of scratch
-cudaError_t exclusive_scan_u32(unsigned* a, long long n, unsigned* sums, cudaStream_t s);
+cudaError_t exclusive_scan_u32(const unsigned* in, unsigned* out, long long n, unsigned* sums, cudaStream_t s);
 // message returned by qc_eloc_last_error(NULL) on this thread (qc_api.cu)
 void set_handleless_error(const std::string& msg);
 // Device allocations of the handle, batch and gradient paths go through here, so that a test

@@ -43,10 +43,13 @@
 
 namespace {
 
-constexpr int kJTile = 2048;  // items per warp tile (64 steps of 32)
 constexpr int kJWarps = 4;    // warps per block (32 KB of per-warp digit counts)
-constexpr int kJBits = 11;
+constexpr int kJBits = 11;    // the widest digit
 constexpr int kJBins = 1 << kJBits;
+
+// Items per tile (one block): a warp ranks its quarter 32 at a time, one step after another, so
+// tables of up to 2.6e5 rows take half-size tiles, whose twice as many blocks still run at once.
+long long tile_items(long long m) { return m <= (1LL << 19) ? 1024 : 2048; }
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -57,7 +60,9 @@ struct JLayout {
 // sort space for m items and n_slots group sizes
 JLayout jlayout(long long m, unsigned long long n_slots) {
     m = std::max<long long>(m, 2);
-    const long long tiles = (m + kJTile - 1) / kJTile;
+    const long long tile = tile_items(m);
+    // (a sort of fewer items, as of the sample order, has no more tiles)
+    const long long tiles = std::max((m + tile - 1) / tile, (std::min<long long>(m, 1LL << 19) + 1023) / 1024);
     const long long table_n = static_cast<long long>(kJBins) * tiles;
     const long long scan_n = std::max<long long>(table_n, static_cast<long long>(n_slots));
     JLayout L{};
@@ -72,19 +77,23 @@ JLayout jlayout(long long m, unsigned long long n_slots) {
     return L;
 }
 
-// One block per tile of kJTile items: the tile's digit counts, table[d * tiles + t].
+// One block per tile: the tile's counts of `bits`-bit digits, table[d * tiles + t].
 __global__ void __launch_bounds__(32 * kJWarps) join_hist_kernel(const unsigned* __restrict__ key, long long m,
-                                                                 int shift, long long tiles,
+                                                                 int shift, int bits, int tile, long long tiles,
                                                                  unsigned* __restrict__ table) {
     __shared__ unsigned hist[kJBins];
-    for (int d = threadIdx.x; d < kJBins; d += blockDim.x) hist[d] = 0u;
+    qc::let_next_start();
+    const int bins = 1 << bits;
+    for (int d = threadIdx.x; d < bins; d += blockDim.x) hist[d] = 0u;
     __syncthreads();
+    qc::wait_previous();
     const long long t = blockIdx.x;
-    const long long i0 = t * kJTile;
-    const long long i1 = i0 + kJTile < m ? i0 + kJTile : m;
-    for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) atomicAdd(&hist[(key[i] >> shift) & (kJBins - 1)], 1u);
+    const long long i0 = t * tile;
+    const long long i1 = i0 + tile < m ? i0 + tile : m;
+#pragma unroll 4
+    for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) atomicAdd(&hist[(key[i] >> shift) & (bins - 1)], 1u);
     __syncthreads();
-    for (int d = threadIdx.x; d < kJBins; d += blockDim.x) table[static_cast<long long>(d) * tiles + t] = hist[d];
+    for (int d = threadIdx.x; d < bins; d += blockDim.x) table[static_cast<long long>(d) * tiles + t] = hist[d];
 }
 
 // Stable scatter of one tile per block: each warp takes a contiguous quarter of the tile,
@@ -96,25 +105,42 @@ __global__ void __launch_bounds__(32 * kJWarps) join_scatter_kernel(const unsign
                                                                     const unsigned* __restrict__ val_in,
                                                                     long long n, unsigned* __restrict__ key_out,
                                                                     unsigned* __restrict__ val_out, long long m,
-                                                                    int shift, long long tiles,
+                                                                    int shift, int bits, int tile, long long tiles,
                                                                     const unsigned* __restrict__ offs) {
-    __shared__ unsigned run[kJWarps][kJBins];
-    constexpr int kSub = kJTile / kJWarps;
+    __shared__ __align__(16) unsigned run[kJWarps][kJBins];
+    // (no let_next_start: a main kernel that becomes resident while this one still holds some SMs
+    // takes 1e5 samples at N=52 from 2.42 to 2.49 ms a step)
+    const int sub = tile / kJWarps, bins = 1 << bits;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long t = blockIdx.x;
-    for (int d = threadIdx.x; d < kJWarps * kJBins; d += blockDim.x) (&run[0][0])[d] = 0u;
+    for (int w = 0; w < kJWarps; ++w)
+        for (int d = threadIdx.x; d < bins; d += blockDim.x) run[w][d] = 0u;
     __syncthreads();
-    const long long i0 = t * kJTile + static_cast<long long>(warp) * kSub;
-    long long i1 = i0 + kSub;
+    qc::wait_previous();
+    const long long i0 = t * tile + static_cast<long long>(warp) * sub;
+    long long i1 = i0 + sub;
     if (i1 > m) i1 = m;
-    for (long long i = i0 + lane; i < i1; i += 32) atomicAdd(&run[warp][(key_in[i] >> shift) & (kJBins - 1)], 1u);
+#pragma unroll 4
+    for (long long i = i0 + lane; i < i1; i += 32) atomicAdd(&run[warp][(key_in[i] >> shift) & (bins - 1)], 1u);
     __syncthreads();
-    for (int d = threadIdx.x; d < kJBins; d += blockDim.x) {
-        unsigned base = offs[static_cast<long long>(d) * tiles + t];
-        for (int w = 0; w < kJWarps; ++w) {
-            const unsigned c = run[w][d];
-            run[w][d] = base;
-            base += c;
+    // the tile's offsets (tiles * 4 bytes apart), eight loads a thread in flight
+    constexpr int kFly = 8;
+    for (int d0 = threadIdx.x; d0 < bins; d0 += kFly * 32 * kJWarps) {
+        unsigned base[kFly];
+#pragma unroll
+        for (int k = 0; k < kFly; ++k) {
+            const int d = d0 + k * 32 * kJWarps;
+            base[k] = d < bins ? offs[static_cast<long long>(d) * tiles + t] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < kFly; ++k) {
+            const int d = d0 + k * 32 * kJWarps;
+            if (d >= bins) break;
+            for (int w = 0; w < kJWarps; ++w) {
+                const unsigned c = run[w][d];
+                run[w][d] = base[k];
+                base[k] += c;
+            }
         }
     }
     __syncthreads();
@@ -126,7 +152,7 @@ __global__ void __launch_bounds__(32 * kJWarps) join_scatter_kernel(const unsign
         if (v) {
             const unsigned k = key_in[i];
             const unsigned val = val_in ? val_in[i] : static_cast<unsigned>(i < n ? i : i - n);
-            const unsigned d = (k >> shift) & (kJBins - 1);
+            const unsigned d = (k >> shift) & (bins - 1);
             const unsigned same = __match_any_sync(active, d);
             const unsigned base = run[warp][d];
             const unsigned pos = base + __popc(same & lt);
@@ -147,6 +173,8 @@ __global__ void __launch_bounds__(256) join_gather_kernel(const ulonglong2* __re
                                                           unsigned set_size, ulonglong2* __restrict__ gent,
                                                           const unsigned* __restrict__ jlen, unsigned* __restrict__ alen,
                                                           unsigned* pa, unsigned* pb) {
+    qc::let_next_start();
+    qc::wait_previous();
     for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < m;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
         const unsigned k = skey[p];
@@ -164,6 +192,8 @@ __global__ void __launch_bounds__(256) join_mark_kernel(const unsigned* __restri
                                                         const unsigned* __restrict__ srow, long long m,
                                                         unsigned set_size, ulonglong2* __restrict__ gent,
                                                         const unsigned* __restrict__ alen) {
+    qc::let_next_start();
+    qc::wait_previous();
     for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < m;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
         const unsigned k = skey[p];
@@ -194,6 +224,8 @@ __global__ void __launch_bounds__(256) join_gather_batch_kernel(const qc::MolPar
                                                                 const unsigned* __restrict__ jlen,
                                                                 unsigned* __restrict__ alen, unsigned* pa,
                                                                 unsigned* pb) {
+    qc::let_next_start();
+    qc::wait_previous();
     const unsigned sentinel = slot_base[n_mol];
     for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < m;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -216,6 +248,8 @@ __global__ void __launch_bounds__(256) join_mark_batch_kernel(const unsigned* __
                                                               ulonglong2* __restrict__ gent,
                                                               const unsigned* __restrict__ row_base,
                                                               const unsigned* __restrict__ alen) {
+    qc::let_next_start();
+    qc::wait_previous();
     const unsigned sentinel = slot_base[n_mol];
     for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < m;
          p += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -241,6 +275,8 @@ __global__ void __launch_bounds__(256) sample_group_sizes_kernel(const qc::Table
                                                                  const unsigned* __restrict__ jlen,
                                                                  unsigned* __restrict__ pa,
                                                                  unsigned* __restrict__ pb) {
+    qc::let_next_start();
+    qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n_u;
          r += static_cast<long long>(gridDim.x) * blockDim.x) {
         const ulonglong2 key = samples[r];
@@ -276,6 +312,8 @@ __device__ __forceinline__ unsigned order_priority_key(unsigned v) {
 __global__ void __launch_bounds__(256) order_key_kernel(const unsigned* __restrict__ pa,
                                                         const unsigned* __restrict__ pb, long long n,
                                                         unsigned* __restrict__ key) {
+    qc::let_next_start();
+    qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
          r += static_cast<long long>(gridDim.x) * blockDim.x)
         key[r] = order_priority_key(pa[r] + pb[r]);
@@ -288,6 +326,8 @@ __global__ void __launch_bounds__(256) order_key_batch_kernel(const unsigned* __
                                                               const unsigned* __restrict__ pa,
                                                               const unsigned* __restrict__ pb, long long n,
                                                               unsigned* __restrict__ key, unsigned* __restrict__ val) {
+    qc::let_next_start();
+    qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
          r += static_cast<long long>(gridDim.x) * blockDim.x) {
         int lo = 0, hi = n_mol;  // largest molecule with row_base <= r
@@ -324,36 +364,43 @@ cudaError_t join_sort(unsigned* jkey, const unsigned* val_in, long long n_half, 
     unsigned* val1 = reinterpret_cast<unsigned*>(W + L.val1);
     unsigned* table = reinterpret_cast<unsigned*>(W + L.table);
     unsigned* sums = reinterpret_cast<unsigned*>(W + L.sums);
-    cudaError_t e = cudaMemcpyAsync(jstart, jlen, n_slots * sizeof(unsigned), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = qc::exclusive_scan_u32(jstart, static_cast<long long>(n_slots), sums, s);
+    cudaError_t e = qc::exclusive_scan_u32(jlen, jstart, static_cast<long long>(n_slots), sums, s);
     if (e == cudaSuccess) e = radix_pairs(jkey, val_in, n_half, m, n_slots, key1, val0, val1, table, sums, skey, sval, s);
     return e;
 }
 
+// One pass: m items by the `bits` bits of their key at `shift`.
+cudaError_t radix_pass(const unsigned* key_in, const unsigned* val_in, long long n_half, long long m, int shift, int bits,
+                       unsigned* key_out, unsigned* val_out, unsigned* table, unsigned* sums, cudaStream_t s) {
+    const int tile = static_cast<int>(tile_items(m));
+    const long long tiles = (m + tile - 1) / tile;
+    const dim3 grid(static_cast<unsigned>(tiles)), block(32 * kJWarps);
+    cudaError_t e = qc::launch_early(join_hist_kernel, grid, block, 0, s, true, key_in, m, shift, bits, tile, tiles, table);
+    if (e == cudaSuccess) e = qc::exclusive_scan_u32(table, table, tiles << bits, sums, s);
+    if (e == cudaSuccess)
+        e = qc::launch_early(join_scatter_kernel, grid, block, 0, s, true, key_in, val_in, n_half, key_out, val_out,
+                             m,
+                             shift, bits, tile, tiles, table);
+    return e;
+}
+
 // Stable LSD sort of m (key, value) items by key (keys up to max_key), values from val_in or
-// (val_in null) the item index modulo n_half; key0 is overwritten (a buffer of the passes).
+// (val_in null) the item index modulo n_half; key0 is overwritten (a buffer of the passes).  The
+// digits share the key's bits evenly, as the counts' table and its scan grow with their width.
 cudaError_t radix_pairs(unsigned* key0, const unsigned* val_in, long long n_half, long long m,
                         unsigned long long max_key, unsigned* key1, unsigned* val0, unsigned* val1,
                         unsigned* table, unsigned* sums, const unsigned** skey, const unsigned** sval,
                         cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     unsigned* jkey = key0;
-    const int passes = (bits_for(max_key) + kJBits - 1) / kJBits;
-    const long long tiles = (m + kJTile - 1) / kJTile;
-    const unsigned blocks = static_cast<unsigned>(tiles);  // one block per tile
+    const int bits = bits_for(max_key);
+    const int passes = (bits + kJBits - 1) / kJBits, width = (bits + passes - 1) / passes;
     const unsigned* src_k = jkey;
     const unsigned* src_v = val_in;
     unsigned* dk[2] = {key1, jkey};
     unsigned* dv[2] = {val0, val1};
     for (int p = 0; p < passes && e == cudaSuccess; ++p) {
-        join_hist_kernel<<<blocks, 32 * kJWarps, 0, s>>>(src_k, m, p * kJBits, tiles, table);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = qc::exclusive_scan_u32(table, static_cast<long long>(kJBins) * tiles, sums, s);
-        if (e == cudaSuccess) {
-            join_scatter_kernel<<<blocks, 32 * kJWarps, 0, s>>>(src_k, src_v, n_half, dk[p & 1], dv[p & 1], m,
-                                                               p * kJBits, tiles, table);
-            e = cudaGetLastError();
-        }
+        e = radix_pass(src_k, src_v, n_half, m, p * width, width, dk[p & 1], dv[p & 1], table, sums, s);
         src_k = dk[p & 1];
         src_v = dv[p & 1];
     }
@@ -378,20 +425,19 @@ cudaError_t qc::launch_join_index(const TableParams& tp, unsigned set_size, void
     const unsigned gblocks = static_cast<unsigned>(std::min<long long>((m + 255) / 256, 8192));
     unsigned* alen = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(ws) + jlayout(m, 2ULL * set_size).alen);
     if (e == cudaSuccess) {
-        join_gather_kernel<<<gblocks, 256, 0, s>>>(tp.keys, skey, sval, m, set_size, gent, jlen, alen,
-                                                   order != nullptr && samples == nullptr ? pa : nullptr, pb);
-        e = cudaGetLastError();
+        e = qc::launch_early(join_gather_kernel, dim3(gblocks), dim3(256), 0, s, true, tp.keys, skey, sval, m,
+                             set_size, gent, jlen, alen, order != nullptr && samples == nullptr ? pa : nullptr, pb);
     }
     if (e == cudaSuccess) {
-        join_mark_kernel<<<gblocks, 256, 0, s>>>(skey, sval, m, set_size, gent, alen);
-        e = cudaGetLastError();
+        e = qc::launch_early(join_mark_kernel, dim3(gblocks), dim3(256), 0, s, true, skey, sval, m, set_size, gent,
+                             alen);
     }
     // the samples to order: the table's rows, or a caller's samples (their groups looked up)
     const long long n = samples != nullptr ? n_samples : tp.n;
     if (e == cudaSuccess && order != nullptr && samples != nullptr && n > 0) {
         const unsigned sblocks = static_cast<unsigned>(std::min<long long>((n + 255) / 256, 8192));
-        sample_group_sizes_kernel<<<sblocks, 256, 0, s>>>(tp, samples, n, T, set_size, jlen, pa, pb);
-        e = cudaGetLastError();
+        e = qc::launch_early(sample_group_sizes_kernel, dim3(sblocks), dim3(256), 0, s, true, tp, samples, n, T,
+                             set_size, jlen, pa, pb);
     }
     if (e == cudaSuccess && order != nullptr && n > 0) {
         // heavy-first sample order: one stable 8-bit pass over the priority keys (the sort
@@ -402,19 +448,9 @@ cudaError_t qc::launch_join_index(const TableParams& tp, unsigned set_size, void
         unsigned* okey2 = reinterpret_cast<unsigned*>(W + L.val0);
         unsigned* table = reinterpret_cast<unsigned*>(W + L.table);
         unsigned* sums = reinterpret_cast<unsigned*>(W + L.sums);
-        order_key_kernel<<<std::min<unsigned>(gblocks, 4096u), 256, 0, s>>>(pa, pb, n, okey);
-        e = cudaGetLastError();
-        const long long tiles = (n + kJTile - 1) / kJTile;
-        const unsigned blocks = static_cast<unsigned>(tiles);  // one block per tile
-        if (e == cudaSuccess) {
-            join_hist_kernel<<<blocks, 32 * kJWarps, 0, s>>>(okey, n, 0, tiles, table);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = qc::exclusive_scan_u32(table, static_cast<long long>(kJBins) * tiles, sums, s);
-        if (e == cudaSuccess) {
-            join_scatter_kernel<<<blocks, 32 * kJWarps, 0, s>>>(okey, nullptr, n, okey2, order, n, 0, tiles, table);
-            e = cudaGetLastError();
-        }
+        e = qc::launch_early(order_key_kernel, dim3(std::min<unsigned>(gblocks, 4096u)), dim3(256), 0, s, true, pa,
+                             pb, n, okey);
+        if (e == cudaSuccess) e = radix_pass(okey, nullptr, n, n, 0, 8, okey2, order, table, sums, s);
     }
     return e;
 }
@@ -432,13 +468,12 @@ cudaError_t qc::launch_join_batch(const MolParams* mols, const unsigned* slot_ba
     const unsigned gblocks = static_cast<unsigned>(std::min<long long>((m + 255) / 256, 8192));
     unsigned* alen = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(ws) + jlayout(m, n_slots).alen);
     if (e == cudaSuccess) {
-        join_gather_batch_kernel<<<gblocks, 256, 0, s>>>(mols, slot_base, n_mol, skey, sval, m, gent, row_base, jlen,
-                                                         alen, order ? pa : nullptr, pb);
-        e = cudaGetLastError();
+        e = qc::launch_early(join_gather_batch_kernel, dim3(gblocks), dim3(256), 0, s, true, mols, slot_base, n_mol,
+                             skey, sval, m, gent, row_base, jlen, alen, order ? pa : nullptr, pb);
     }
     if (e == cudaSuccess) {
-        join_mark_batch_kernel<<<gblocks, 256, 0, s>>>(slot_base, n_mol, skey, sval, m, gent, row_base, alen);
-        e = cudaGetLastError();
+        e = qc::launch_early(join_mark_batch_kernel, dim3(gblocks), dim3(256), 0, s, true, slot_base, n_mol, skey,
+                             sval, m, gent, row_base, alen);
     }
     if (e == cudaSuccess && order != nullptr) {
         // every joining molecule's rows heavy first: keys and values into the sort's input
@@ -446,9 +481,8 @@ cudaError_t qc::launch_join_batch(const MolParams* mols, const unsigned* slot_ba
         const long long R = m / 2;
         const JLayout L = jlayout(m, n_slots);
         unsigned char* W = static_cast<unsigned char*>(ws);
-        order_key_batch_kernel<<<std::min<unsigned>(gblocks, 4096u), 256, 0, s>>>(row_base, n_mol, pa, pb, R, jkey,
-                                                                                 jval);
-        e = cudaGetLastError();
+        e = qc::launch_early(order_key_batch_kernel, dim3(std::min<unsigned>(gblocks, 4096u)), dim3(256), 0, s, true,
+                             row_base, n_mol, pa, pb, R, jkey, jval);
         if (e == cudaSuccess)
             e = radix_pairs(jkey, jval, R, R, (static_cast<unsigned long long>(n_mol) << 8) | 255ULL,
                             reinterpret_cast<unsigned*>(W + L.key1), reinterpret_cast<unsigned*>(W + L.val0),

@@ -11,24 +11,6 @@
 
 namespace qc {
 
-// Launch with programmatic stream serialization (early) or plainly: the kernel may start while the
-// stream's previous kernel runs and synchronises with it by wait_previous.
-template <typename... P, typename... A>
-static cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool early,
-                                A... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 template <int PREC, int U, bool FILTER, int LEAN, bool JOIN, bool DIAG, bool SEG = false>
 __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const __grid_constant__ SysParams sp,
                                                         const __grid_constant__ TableParams tp,
@@ -100,6 +82,15 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
     }
 }
 
+// Threads of a CTA: the shape's warps, or just enough for the items when those are fewer than the
+// grid's warps, so that every CTA gets as many (with all warps started, first come took 60 us in
+// the place of 56 for 1,000 samples at N=14).
+static dim3 main_block(const EvalParams& ep, const LaunchCfg& c) {
+    const long long items = ep.n_u * (ep.chunks > 1 ? ep.chunks : 1);
+    const long long w = (items + c.grid - 1) / c.grid;
+    return dim3(32 * static_cast<unsigned>(w < 1 ? 1 : w < c.warps ? w : c.warps));
+}
+
 template <int PREC, int LEAN, bool DIAG>
 static cudaError_t launch_filtered(const SysParams& sp, const TableParams& tp, const EvalParams& ep, const LaunchCfg& c,
                                    cudaStream_t s) {
@@ -108,14 +99,14 @@ static cudaError_t launch_filtered(const SysParams& sp, const TableParams& tp, c
     else if (c.join) k = eloc_main_kernel<PREC, 4, true, LEAN, true, DIAG>;
     else if (c.unroll == 1) k = eloc_main_kernel<PREC, 1, true, LEAN, false, DIAG>;
     else if (c.unroll == 2) k = eloc_main_kernel<PREC, 2, true, LEAN, false, DIAG>;
-    return launch_early(k, dim3(c.grid), dim3(32 * c.warps), c.smem, s, c.early != 0, sp, tp, ep);
+    return launch_early(k, dim3(c.grid), main_block(ep, c), c.smem, s, c.early != 0, sp, tp, ep);
 }
 
 template <int PREC, bool DIAG>
 static cudaError_t launch_main_p(const SysParams& sp, const TableParams& tp, const EvalParams& ep,
                                  const LaunchCfg& c, cudaStream_t s) {
     if (c.kernel != 2)
-        return launch_early(eloc_main_kernel<PREC, 1, false, 0, false, DIAG>, dim3(c.grid), dim3(32 * c.warps), c.smem, s,
+        return launch_early(eloc_main_kernel<PREC, 1, false, 0, false, DIAG>, dim3(c.grid), main_block(ep, c), c.smem, s,
                             c.early != 0, sp, tp, ep);
     return c.lean ? launch_filtered<PREC, 1, DIAG>(sp, tp, ep, c, s) : launch_filtered<PREC, 0, DIAG>(sp, tp, ep, c, s);
 }
