@@ -862,7 +862,7 @@ __device__ __forceinline__ bool sample_setup(const SysParams& sp, ulonglong2 x, 
 }
 
 // Lane 0's part of a sample's finish: E_loc from the warp sums and the outputs.
-template <int PREC>
+template <int PREC, bool DIAG>
 __device__ __forceinline__ void write_sample(const EvalParams& ep, long long s, double ediag, double2 psix,
                                              double sre, double sim, unsigned long long hits,
                                              unsigned long long rows, long long sgn, unsigned long long miss) {
@@ -891,9 +891,11 @@ __device__ __forceinline__ void write_sample(const EvalParams& ep, long long s, 
         e.y = sim;
     }
     ep.eloc[QC_IX(s, ep.n_u, &ep.ctr->flags)] = e;
-    if (ep.hit_count) ep.hit_count[s] = static_cast<uint32_t>(hits);
-    if (ep.hit_rowsum) ep.hit_rowsum[s] = rows;
-    if (ep.hit_signsum) ep.hit_signsum[s] = sgn;
+    if (DIAG) {  // (asked for, these outputs take the diagnostic kernels)
+        if (ep.hit_count) ep.hit_count[s] = static_cast<uint32_t>(hits);
+        if (ep.hit_rowsum) ep.hit_rowsum[s] = rows;
+        if (ep.hit_signsum) ep.hit_signsum[s] = sgn;
+    }
     if (hits) atomicAdd(&ep.ctr->hits, hits);
     if (miss) atomicAdd(&ep.ctr->missing, miss);
     if (bad) atomicAdd(&ep.ctr->bad, 1ULL);
@@ -901,7 +903,7 @@ __device__ __forceinline__ void write_sample(const EvalParams& ep, long long s, 
 }
 
 // One chunk of a sample evaluated in C > 1 excitation chunks (out of line: off by default).
-template <int PREC>
+template <int PREC, bool DIAG>
 static __device__ __noinline__ void finish_chunk(const EvalParams& ep, long long s, double ediag, double2 psix,
                                                  const ChunkRec& mine, int c, int C) {
     ChunkRec* rec = static_cast<ChunkRec*>(ep.cpart) + s * C;
@@ -921,7 +923,7 @@ static __device__ __noinline__ void finish_chunk(const EvalParams& ep, long long
         ts += r->signsum;
         tm += r->missing;
     }
-    write_sample<PREC>(ep, s, ediag, psix, re, im, th, tr, ts, tm);
+    write_sample<PREC, DIAG>(ep, s, ediag, psix, re, im, th, tr, ts, tm);
 }
 
 // Per-sample finish: reduce the lane accumulators and write the outputs.  With several
@@ -947,7 +949,7 @@ __device__ __forceinline__ void sample_finish(const EvalParams& ep, long long s,
     const unsigned long long miss = FILTER ? 0ULL : warp_sum_u64(acc.missing);
     if (lane != 0) return;
     if (C <= 1) {
-        write_sample<PREC>(ep, s, ediag, psix, sre, sim, hits, rows, sgn, miss);
+        write_sample<PREC, DIAG>(ep, s, ediag, psix, sre, sim, hits, rows, sgn, miss);
         return;
     }
     ChunkRec mine;
@@ -957,7 +959,7 @@ __device__ __forceinline__ void sample_finish(const EvalParams& ep, long long s,
     mine.rowsum = rows;
     mine.signsum = sgn;
     mine.missing = miss;
-    finish_chunk<PREC>(ep, s, ediag, psix, mine, c, C);
+    finish_chunk<PREC, DIAG>(ep, s, ediag, psix, mine, c, C);
 }
 
 static __device__ __noinline__ void invalid_sample(const EvalParams& ep, long long s, int lane) {

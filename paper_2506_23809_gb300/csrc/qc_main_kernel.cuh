@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
         if (lane == 0) it = atomicAdd(&ep.ctr->next, 1ULL);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= items) break;
-        const unsigned long long q = it / C;
+        const unsigned long long q = C == 1 ? it : it / C;
         // heavy samples first when the host gave an order: the launch then ends on light ones
         const unsigned long long s =
             ep.order != nullptr ? static_cast<unsigned long long>(__ldg(ep.order + QC_IX(q, ep.n_u, sp.err))) : q;
