@@ -17,7 +17,7 @@
 // spin-string sets as a sort key (alpha rows first, beta rows offset by the set size) and
 // the group sizes:
 //   starts:    exclusive prefix sum of the group sizes
-//   J1 hist:   per-tile digit counts (11-bit digits of the slot key)
+//   J1 hist:   per-tile digit counts (digits of up to 11 bits that share the slot key evenly)
 //   scan:      exclusive prefix over the (digit, tile) counts, digit-major
 //   J2 scatter: stable scatter of (key, row) by digit; after the passes the pairs are in
 //              (slot, row) order, so every group lists its rows in row order and the scan
@@ -30,8 +30,10 @@
 //              bits (the kernel's scan of a beta' group keeps the rows of long alpha' groups
 //              by it, without a lookup)
 // Traffic per row: 8 B read (hist) + 8 B read + 8 B written (scatter) per pass and key half,
-// then 16 B read, 16 B written (gather) and 12 B read, 8 B written (mark); a few tens of
-// microseconds at 10^5 rows.
+// then 16 B read, 16 B written (gather) and 12 B read, 8 B written (mark).  Bound by the latency
+// of some twenty dependent kernels: digits no wider than the key needs, 1,024-item tiles, eight
+// offset loads in flight and programmatic dependent launch took an evaluation of 4,953 rows at
+// N=106 from 585 to 518 us and of 10^5 rows at N=52 from 2.46 to 2.42 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
