@@ -10,7 +10,7 @@
 // coalesced along a row): 0.97 ms for 1e5 x 4,096 at the 6.78 TB/s of a copy.  Two FP64
 // fused multiply-adds per element would take 1.38 ms (the FP64 pipe retires two per clock and
 // SM), so the real parts go through that pipe and the imaginary parts through integer
-// multiplications (FixedSum), which run beside it: 1.44 -> 1.01 ms a call, 6.5 TB/s.
+// multiplications (FixedSum), which run beside it: 1.44 -> 1.00 ms a call, 6.6 TB/s.
 #include <cuda_runtime.h>
 
 #include <algorithm>
