@@ -556,8 +556,8 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* s
     return before + x - v;
 }
 
-__global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const unsigned* __restrict__ a, long long n,
-                                                               unsigned* __restrict__ sums) {
+__global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const unsigned* a, long long n,
+                                                               unsigned* sums) {
     __shared__ unsigned sh[32];
     qc::let_next_start();
     qc::wait_previous();
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kScanBlock) scan_sums_kernel(const unsigned* _
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__device__ __forceinline__ void scan_top(unsigned* __restrict__ sums, long long m) {
+__device__ __forceinline__ void scan_top(unsigned* sums, long long m) {
     __shared__ unsigned sh[32];
     __shared__ unsigned carry;
     if (threadIdx.x == 0) carry = 0;
@@ -589,7 +589,7 @@ __device__ __forceinline__ void scan_top(unsigned* __restrict__ sums, long long 
     if (threadIdx.x == 0) sums[m] = carry;
 }
 
-__global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* __restrict__ sums, long long m) {
+__global__ void __launch_bounds__(kScanBlock) scan_top_kernel(unsigned* sums, long long m) {
     qc::let_next_start();
     qc::wait_previous();
     scan_top(sums, m);
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(kScanBlock) dedup_scan_kernel(unsigned* __rest
 }
 
 __global__ void __launch_bounds__(kScanBlock) scan_down_kernel(const unsigned* a, unsigned* out, long long n,
-                                                               const unsigned* __restrict__ sums) {
+                                                               const unsigned* sums) {
     __shared__ unsigned sh[32];
     qc::let_next_start();
     qc::wait_previous();

@@ -158,6 +158,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -189,7 +190,7 @@ __device__ __forceinline__ long long table_find(const TableParams& tp, ulonglong
     const ulonglong2* buckets = reinterpret_cast<const ulonglong2*>(tp.slots);
 #pragma unroll 1
     for (unsigned it = 0; it <= tp.nb_mask; ++it) {
-        const ulonglong2 e = __ldg(buckets + QC_IX(b, tp.nb_mask + 1LL, tp.err));
+        const ulonglong2 e = buckets[QC_IX(b, tp.nb_mask + 1LL, tp.err)];
         if (e.x == 0ULL) return -1;
         if (static_cast<unsigned>(e.x >> 32) == g) {
             const long long r = static_cast<long long>(static_cast<unsigned>(e.x)) - 1;
@@ -215,7 +216,7 @@ __device__ __forceinline__ long long probe_fp(unsigned g, const TableParams& tp)
     const ulonglong2* buckets = reinterpret_cast<const ulonglong2*>(tp.slots);
 #pragma unroll 1
     for (unsigned it = 0; it <= tp.nb_mask; ++it) {
-        const ulonglong2 e = __ldg(buckets + QC_IX(b, tp.nb_mask + 1LL, tp.err));
+        const ulonglong2 e = buckets[QC_IX(b, tp.nb_mask + 1LL, tp.err)];
         if (e.x == 0ULL) return -1;
         if (static_cast<unsigned>(e.x >> 32) == g) return static_cast<long long>(static_cast<unsigned>(e.x)) - 1;
         if (e.y == 0ULL) return -1;
@@ -249,12 +250,12 @@ __device__ __forceinline__ unsigned set_insert(unsigned long long* set, unsigned
 }
 
 // The slot that holds spin string v, or kNoSlot.
-__device__ __forceinline__ unsigned set_slot(const unsigned long long* __restrict__ set, unsigned mask,
-                                             unsigned long long v, unsigned long long h) {
+__device__ __forceinline__ unsigned set_slot(const unsigned long long* set, unsigned mask, unsigned long long v,
+                                             unsigned long long h) {
     unsigned b = static_cast<unsigned>(h >> 32) & mask;
 #pragma unroll 1
     for (unsigned it = 0; it <= mask; ++it) {
-        const unsigned long long e = __ldg(set + (b & mask));
+        const unsigned long long e = set[b & mask];
         if (e == v) return b;
         if (e == 0ULL) return kNoSlot;
         b = (b + 1u) & mask;
@@ -262,7 +263,7 @@ __device__ __forceinline__ unsigned set_slot(const unsigned long long* __restric
     return kNoSlot;
 }
 
-__device__ __forceinline__ bool set_contains(const unsigned long long* __restrict__ set, unsigned mask,
+__device__ __forceinline__ bool set_contains(const unsigned long long* set, unsigned mask,
                                              unsigned long long v, unsigned long long h) {
     return set_slot(set, mask, v, h) != kNoSlot;
 }
@@ -1266,12 +1267,12 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
                 const unsigned off = lane == 0 ? 0u : tp.set_mask + 1u;
                 const unsigned sl = lane == 0 ? set_slot(tp.aset, tp.set_mask, As, hxa)
                                               : set_slot(tp.bset, tp.set_mask, Bs, hxb);
-                const unsigned len = sl != kNoSlot ? __ldg(tp.jlen + QC_IX(off + sl, 2LL * (tp.set_mask + 1LL), tp.err)) : 0u;
+                const unsigned len = sl != kNoSlot ? tp.jlen[QC_IX(off + sl, 2LL * (tp.set_mask + 1LL), tp.err)] : 0u;
                 const long long pairs = lane == 0 ? static_cast<long long>(nsb2) + static_cast<long long>(sp.npob) * sp.npvb
                                                   : static_cast<long long>(sp.npoa) * sp.npva;
                 if (len > 0u) {
                     if (static_cast<long long>(len) * tp.scan_cost <= 4 * pairs) {
-                        gst = __ldg(tp.jstart + QC_IX(off + sl, 2LL * (tp.set_mask + 1LL), tp.err));
+                        gst = tp.jstart[QC_IX(off + sl, 2LL * (tp.set_mask + 1LL), tp.err)];
                         gln = len;
                     } else {
                         en = true;
@@ -1404,7 +1405,7 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
                     unsigned code = 0u, row = 0u;
                     if (v < stotal) {
                         const unsigned kd = q[64 + g];
-                        const ulonglong2 e = __ldg(tp.gent + QC_IX(q[g] + (v - q[32 + g]), 2 * tp.n, tp.err));
+                        const ulonglong2 e = tp.gent[QC_IX(q[g] + (v - q[32 + g]), 2 * tp.n, tp.err)];
                         const unsigned kk = kd & 3u;
                         const unsigned long long ref = (BETA ? (kk & 1u) == 0u : kk == kScanBeta) ? ras : rbs;
                         const unsigned long long dm = e.x ^ ref;
@@ -1454,8 +1455,8 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
                     hv32 = static_cast<uint32_t>(tm);
                     const unsigned sl = set_slot(tp.aset, tp.set_mask, wsp->as ^ (1ULL << ki) ^ (1ULL << ka), wsp->hxa ^ tm);
                     if (sl != kNoSlot) {
-                        len = __ldg(tp.jlen + QC_IX(sl, tp.set_mask + 1LL, tp.err));
-                        start = __ldg(tp.jstart + QC_IX(sl, tp.set_mask + 1LL, tp.err));
+                        len = tp.jlen[QC_IX(sl, tp.set_mask + 1LL, tp.err)];
+                        start = tp.jstart[QC_IX(sl, tp.set_mask + 1LL, tp.err)];
                     }
                     lng = BETA ? len > wsp->athr : static_cast<long long>(len) * tp.scan_cost > 4LL * (nsb2 + 1);
                     kd = kScanAlphaP | (static_cast<unsigned>(ki) << 8) | (static_cast<unsigned>(ka) << 16);
@@ -1515,10 +1516,10 @@ __device__ __forceinline__ void run_sample(const SysParams& sp, const TableParam
                                                  wsp->hx ^ wsp->hxa ^ tm);
                     const long long jo = static_cast<long long>(tp.set_mask) + 1LL + sl;
                     const unsigned len =
-                        sl != kNoSlot ? __ldg(tp.jlen + QC_IX(jo, 2LL * (tp.set_mask + 1LL), tp.err)) : 0u;
+                        sl != kNoSlot ? tp.jlen[QC_IX(jo, 2LL * (tp.set_mask + 1LL), tp.err)] : 0u;
                     keep = !(len > 0u && static_cast<long long>(len) * tp.beta_cost <= 4LL * nsa2);
                     if (!keep) {
-                        gst = __ldg(tp.jstart + QC_IX(jo, 2LL * (tp.set_mask + 1LL), tp.err));
+                        gst = tp.jstart[QC_IX(jo, 2LL * (tp.set_mask + 1LL), tp.err)];
                         gln = len;
                         // bit 2: x's beta single is taken from the group (class 1 is enumerated)
                         kd = kScanBetaP | (enumA ? 4u : 0u) | (kj << 8) | (kb << 16);

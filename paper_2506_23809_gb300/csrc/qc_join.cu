@@ -80,9 +80,9 @@ JLayout jlayout(long long m, unsigned long long n_slots) {
 }
 
 // One block per tile: the tile's counts of `bits`-bit digits, table[d * tiles + t].
-__global__ void __launch_bounds__(32 * kJWarps) join_hist_kernel(const unsigned* __restrict__ key, long long m,
+__global__ void __launch_bounds__(32 * kJWarps) join_hist_kernel(const unsigned* key, long long m,
                                                                  int shift, int bits, int tile, long long tiles,
-                                                                 unsigned* __restrict__ table) {
+                                                                 unsigned* table) {
     __shared__ unsigned hist[kJBins];
     qc::let_next_start();
     const int bins = 1 << bits;
@@ -103,12 +103,12 @@ __global__ void __launch_bounds__(32 * kJWarps) join_hist_kernel(const unsigned*
 // tile order); then every warp walks its quarter in index order (__match_any_sync ranks
 // equal digits within a step of 32).  The first pass takes the row from the index (item
 // i < n is row i's alpha key, item n + i its beta key).
-__global__ void __launch_bounds__(32 * kJWarps) join_scatter_kernel(const unsigned* __restrict__ key_in,
-                                                                    const unsigned* __restrict__ val_in,
-                                                                    long long n, unsigned* __restrict__ key_out,
-                                                                    unsigned* __restrict__ val_out, long long m,
+__global__ void __launch_bounds__(32 * kJWarps) join_scatter_kernel(const unsigned* key_in,
+                                                                    const unsigned* val_in,
+                                                                    long long n, unsigned* key_out,
+                                                                    unsigned* val_out, long long m,
                                                                     int shift, int bits, int tile, long long tiles,
-                                                                    const unsigned* __restrict__ offs) {
+                                                                    const unsigned* offs) {
     __shared__ __align__(16) unsigned run[kJWarps][kJBins];
     // (no let_next_start: a main kernel that becomes resident while this one still holds some SMs
     // takes 1e5 samples at N=52 from 2.42 to 2.49 ms a step)
@@ -170,10 +170,10 @@ __global__ void __launch_bounds__(32 * kJWarps) join_scatter_kernel(const unsign
 // (alen: each row's alpha-group size, from its alpha entry; with pa: each row's own alpha-
 // and beta-group sizes into pa / pb, for the sample order)
 __global__ void __launch_bounds__(256) join_gather_kernel(const ulonglong2* __restrict__ keys,
-                                                          const unsigned* __restrict__ skey,
-                                                          const unsigned* __restrict__ srow, long long m,
-                                                          unsigned set_size, ulonglong2* __restrict__ gent,
-                                                          const unsigned* __restrict__ jlen, unsigned* __restrict__ alen,
+                                                          const unsigned* skey,
+                                                          const unsigned* srow, long long m,
+                                                          unsigned set_size, ulonglong2* gent,
+                                                          const unsigned* jlen, unsigned* alen,
                                                           unsigned* pa, unsigned* pb) {
     qc::let_next_start();
     qc::wait_previous();
@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(256) join_gather_kernel(const ulonglong2* __re
 }
 
 // J4: the beta entries' row words get the row's alpha-group size in their high half.
-__global__ void __launch_bounds__(256) join_mark_kernel(const unsigned* __restrict__ skey,
-                                                        const unsigned* __restrict__ srow, long long m,
-                                                        unsigned set_size, ulonglong2* __restrict__ gent,
-                                                        const unsigned* __restrict__ alen) {
+__global__ void __launch_bounds__(256) join_mark_kernel(const unsigned* skey,
+                                                        const unsigned* srow, long long m,
+                                                        unsigned set_size, ulonglong2* gent,
+                                                        const unsigned* alen) {
     qc::let_next_start();
     qc::wait_previous();
     for (long long p = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; p < m;
@@ -219,12 +219,12 @@ __device__ __forceinline__ int batch_molecule(const unsigned* __restrict__ slot_
 // key, then the sentinel), the spin from the key's place in the molecule's two sets.
 __global__ void __launch_bounds__(256) join_gather_batch_kernel(const qc::MolParams* __restrict__ mols,
                                                                 const unsigned* __restrict__ slot_base, int n_mol,
-                                                                const unsigned* __restrict__ skey,
-                                                                const unsigned* __restrict__ srow, long long m,
-                                                                ulonglong2* __restrict__ gent,
+                                                                const unsigned* skey,
+                                                                const unsigned* srow, long long m,
+                                                                ulonglong2* gent,
                                                                 const unsigned* __restrict__ row_base,
-                                                                const unsigned* __restrict__ jlen,
-                                                                unsigned* __restrict__ alen, unsigned* pa,
+                                                                const unsigned* jlen,
+                                                                unsigned* alen, unsigned* pa,
                                                                 unsigned* pb) {
     qc::let_next_start();
     qc::wait_previous();
@@ -245,11 +245,11 @@ __global__ void __launch_bounds__(256) join_gather_batch_kernel(const qc::MolPar
 
 // J4 of a batch: the beta entries' row words get the row's alpha-group size.
 __global__ void __launch_bounds__(256) join_mark_batch_kernel(const unsigned* __restrict__ slot_base, int n_mol,
-                                                              const unsigned* __restrict__ skey,
-                                                              const unsigned* __restrict__ srow, long long m,
-                                                              ulonglong2* __restrict__ gent,
+                                                              const unsigned* skey,
+                                                              const unsigned* srow, long long m,
+                                                              ulonglong2* gent,
                                                               const unsigned* __restrict__ row_base,
-                                                              const unsigned* __restrict__ alen) {
+                                                              const unsigned* alen) {
     qc::let_next_start();
     qc::wait_previous();
     const unsigned sentinel = slot_base[n_mol];
@@ -274,9 +274,9 @@ __global__ void __launch_bounds__(256) sample_group_sizes_kernel(const qc::Table
                                                                  long long n_u,
                                                                  const unsigned long long* __restrict__ T,
                                                                  unsigned set_size,
-                                                                 const unsigned* __restrict__ jlen,
-                                                                 unsigned* __restrict__ pa,
-                                                                 unsigned* __restrict__ pb) {
+                                                                 const unsigned* jlen,
+                                                                 unsigned* pa,
+                                                                 unsigned* pb) {
     qc::let_next_start();
     qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n_u;
@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(256) sample_group_sizes_kernel(const qc::Table
         const unsigned long long sa = qc::spin_string(key, 0), sb = qc::spin_string(key, 1);
         const unsigned la = sa != 0ULL ? qc::set_slot(tp.aset, tp.set_mask, sa, ha) : qc::kNoSlot;
         const unsigned lb = sb != 0ULL ? qc::set_slot(tp.bset, tp.set_mask, sb, hb) : qc::kNoSlot;
-        pa[r] = la != qc::kNoSlot ? __ldg(jlen + la) : 0u;
-        pb[r] = lb != qc::kNoSlot ? __ldg(jlen + set_size + lb) : 0u;
+        pa[r] = la != qc::kNoSlot ? jlen[la] : 0u;
+        pb[r] = lb != qc::kNoSlot ? jlen[set_size + lb] : 0u;
     }
 }
 
@@ -311,9 +311,9 @@ __device__ __forceinline__ unsigned order_priority_key(unsigned v) {
     return 255u - (bucket > 255u ? 255u : bucket);
 }
 
-__global__ void __launch_bounds__(256) order_key_kernel(const unsigned* __restrict__ pa,
-                                                        const unsigned* __restrict__ pb, long long n,
-                                                        unsigned* __restrict__ key) {
+__global__ void __launch_bounds__(256) order_key_kernel(const unsigned* pa,
+                                                        const unsigned* pb, long long n,
+                                                        unsigned* key) {
     qc::let_next_start();
     qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n;
@@ -325,9 +325,9 @@ __global__ void __launch_bounds__(256) order_key_kernel(const unsigned* __restri
 // index << 8 | priority, value = the row within its molecule, so one stable sort gives every
 // molecule's rows heavy first, molecule after molecule.
 __global__ void __launch_bounds__(256) order_key_batch_kernel(const unsigned* __restrict__ row_base, int n_mol,
-                                                              const unsigned* __restrict__ pa,
-                                                              const unsigned* __restrict__ pb, long long n,
-                                                              unsigned* __restrict__ key, unsigned* __restrict__ val) {
+                                                              const unsigned* pa,
+                                                              const unsigned* pb, long long n,
+                                                              unsigned* key, unsigned* val) {
     qc::let_next_start();
     qc::wait_previous();
     for (long long r = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; r < n;

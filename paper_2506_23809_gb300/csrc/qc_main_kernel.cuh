@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
         if (threadIdx.x == 0) {
             mbar_init(bar, 1);
             fence_barrier_init();
+            fence_async_global();  // the filter's words were written by ordinary stores of this chain
         }
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(32 * kFilteredMaxWarps) eloc_main_kernel(const
         const unsigned long long q = C == 1 ? it : it / C;
         // heavy samples first when the host gave an order: the launch then ends on light ones
         const unsigned long long s =
-            ep.order != nullptr ? static_cast<unsigned long long>(__ldg(ep.order + QC_IX(q, ep.n_u, sp.err))) : q;
+            ep.order != nullptr ? static_cast<unsigned long long>(ep.order[QC_IX(q, ep.n_u, sp.err)]) : q;
         run_sample<PREC, U, FILTER, LEAN, JOIN, DIAG, SEG, SEG>(sp, tp, ep, static_cast<long long>(s), lane, smem, wl, filt,
                                                 static_cast<int>(it - q * C), static_cast<int>(C));
     }
