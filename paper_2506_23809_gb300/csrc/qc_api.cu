@@ -204,6 +204,7 @@ qc_status qc_eloc_create(const double* h, const double* eri, double e_core, int 
     QC_TRY(qc::dev_alloc(&H->d_sum, sizeof(qc_eloc_summary)), "cudaMalloc summary");
     if (H->device >= 0 && H->device < 64 && !prepared_devices[H->device]) {
         QC_TRY(qc::prepare_kernels(H->smem_optin), "cudaFuncSetAttribute");
+        QC_TRY(qc::prepare_export(), "cudaFuncSetAttribute");
         prepared_devices[H->device] = true;
     }
 #undef QC_TRY

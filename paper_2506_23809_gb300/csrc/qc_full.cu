@@ -77,6 +77,7 @@ constexpr size_t kExpOffList = kOffVar;
 constexpr size_t kExpOffU = kExpOffList + 256;
 constexpr size_t kExpOffW = kExpOffU + kExpUTile * sizeof(ExpU);
 inline size_t export_smem_bytes(const SysParams& sp) { return kExpOffW + static_cast<size_t>(exp_max_w(sp)) * (16 + 4); }
+constexpr size_t kExpSmemMax = kExpOffW + kPairLut * (16 + 4);  // a spin's 64 orbitals all empty: 2,016 pairs
 
 __device__ __forceinline__ ulonglong2 key_bits(int p, int q) {
     ulonglong2 k = make_ulonglong2(0ULL, 0ULL);
@@ -457,6 +458,21 @@ qc_status ffail(qc_eloc* H, qc_status st, const std::string& m) {
 }
 
 }  // namespace
+
+// The export kernels' shared-memory limit belongs to the function, not to a launch: it is set once,
+// to the most any handle needs (set per call to the handle's own size, threads exporting with
+// different handles lowered it between each other's call and launch).
+cudaError_t prepare_export() {
+    cudaError_t e = cudaSuccess;
+    for (const void* f : {(const void*)eloc_export_kernel<QC_FP64, 128>, (const void*)eloc_export_kernel<QC_FP32_COMP, 128>,
+                          (const void*)eloc_export_kernel<QC_FP64, 256>, (const void*)eloc_export_kernel<QC_FP32_COMP, 256>}) {
+        const cudaError_t r =
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kExpSmemMax));
+        if (r != cudaSuccess) e = r;
+    }
+    return e;
+}
+
 }  // namespace qc
 
 extern "C" qc_status qc_eloc_export(qc_eloc* H, const uint64_t* samples, int64_t n_u, uint64_t* keys_out,
@@ -483,10 +499,8 @@ extern "C" qc_status qc_eloc_export(qc_eloc* H, const uint64_t* samples, int64_t
     const int T = H->sp.pairs < 8192 ? 128 : 256;
     const Kernel f = T == 128 ? (f64 ? qc::eloc_export_kernel<QC_FP64, 128> : qc::eloc_export_kernel<QC_FP32_COMP, 128>)
                               : (f64 ? qc::eloc_export_kernel<QC_FP64, 256> : qc::eloc_export_kernel<QC_FP32_COMP, 256>);
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, T, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, T, smem);
     if (e != cudaSuccess || per_sm < 1)
         return qc::ffail(H, QC_ERR_CUDA, std::string("export: ") + cudaGetErrorString(e));
     // pairs per work item: about kExpItemPairs, fewer when that leaves the chip's CTAs short of work

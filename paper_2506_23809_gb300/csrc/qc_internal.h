@@ -293,6 +293,7 @@ int max_active_batch(int precision, int unroll, int threads, size_t smem, bool j
 size_t batch_warp_bytes(const SysParams& sp, bool lean, bool join, int acap);
 cudaError_t prepare_batch_kernels(size_t max_smem, size_t* dyn_limit);
 cudaError_t prepare_kernels(size_t max_smem);
+cudaError_t prepare_export();  // qc_full.cu
 size_t filtered_smem_bytes(const SysParams& sp, int warps, int fw, bool lean = false, bool join = false, int acap = 0);
 size_t direct_smem_bytes(const SysParams& sp, int warps);
 size_t smem_fixed_bytes();  // CTA tables at the head of the main kernels' dynamic shared memory
