@@ -224,9 +224,10 @@ __global__ void __launch_bounds__(32 * kFinishGroups) grad_finish_kernel(const d
 // The contraction's split: columns per CTA (256 >> shift), rows per chunk and chunks.  A function
 // of the sizes only (not of the GPU), so the summation order, and the result, are the same
 // everywhere.  Up to 128 columns the CTA's threads share the rows; the chunks fill whole waves of
-// kGradWave CTAs (four on each of 152 SMs) with at most 256 rows a CTA and at least 8 a thread,
-// as a CTA starts and ends with some twenty FP64 operations a thread (5,723 x 2,816: 64-row
-// chunks of 256 columns 80 us, of 32 columns 126 us).
+// kGradWave CTAs (four on each of 152 SMs) with at most 256 rows a CTA (more only beyond
+// kGradChunksMax x 256 rows) and at least 8 a thread, as a CTA starts and ends with some twenty
+// FP64 operations a thread (5,723 x 2,816: 64-row chunks of 256 columns 80 us, of 32 columns
+// 126 us).
 constexpr long long kGradWave = 608, kGradChunksMax = 512;
 struct GradSplit {
     int shift, chunks;
@@ -244,6 +245,11 @@ GradSplit grad_split(long long n, long long P) {
     g.chunks = static_cast<int>((n + g.rows - 1) / g.rows);
     return g;
 }
+
+// The most chunks that a call of up to n rows splits into, whatever its columns: the partials'
+// buffer is sized by it, so that a later call that is no larger in rows and columns fits (the
+// split itself is not monotone: 2,433 x 300 has 271 chunks, 2,432 x 300 has 304).
+long long grad_chunks_bound(long long n) { return std::min<long long>(kGradChunksMax, (n + 7) / 8); }
 
 }  // namespace
 
@@ -280,7 +286,7 @@ extern "C" qc_status qc_eloc_grad(qc_eloc* H, const double* eloc, const int64_t*
         } else {
             const GradSplit sp = grad_split(n_u, n_par);
             const int chunks = sp.chunks;
-            const size_t need = static_cast<size_t>(chunks) * static_cast<size_t>(n_par);
+            const size_t need = static_cast<size_t>(grad_chunks_bound(n_u)) * static_cast<size_t>(n_par);
             if (need > H->gpart_cap) {
                 if (H->d_gpart) cudaFree(H->d_gpart);
                 H->d_gpart = nullptr;
