@@ -44,14 +44,14 @@ __global__ void __launch_bounds__(256) grad_weights_kernel(const double2* __rest
 
 // One staged row: its weight, and the imaginary weight's mantissa (the leading bit at bit 63),
 // biased exponent and the sign of -w.y as a mask.  A weight that is zero, subnormal or not
-// finite has an exponent that puts each of its products out of FixedSum's window.
+// finite has an exponent of its own that puts each of its products out of FixedSum's window.
 struct __align__(16) GradRow {
     double2 w;
     unsigned mhi, mlo;
     int ex;
     unsigned neg;
 };
-constexpr int kNoExponent = 1 << 20;
+constexpr int kNotFinite = 1 << 20, kSubnormal = -kNotFinite, kZero = -2 * kNotFinite;
 
 __device__ __forceinline__ GradRow grad_row(double2 w) {
     const unsigned hi = static_cast<unsigned>(__double2hiint(w.y)), lo = static_cast<unsigned>(__double2loint(w.y));
@@ -60,7 +60,7 @@ __device__ __forceinline__ GradRow grad_row(double2 w) {
     r.w = w;
     r.mhi = 0x80000000u | __funnelshift_l(lo, hi, 11);
     r.mlo = lo << 11;
-    r.ex = ex == 0 ? -kNoExponent : ex == 0x7ff ? kNoExponent : ex;
+    r.ex = ex == 0 ? (w.y == 0.0 ? kZero : kSubnormal) : ex == 0x7ff ? kNotFinite : ex;
     r.neg = static_cast<unsigned>(~static_cast<int>(hi) >> 31);
     return r;
 }
@@ -70,23 +70,25 @@ __device__ __forceinline__ GradRow grad_row(double2 w) {
 // relative), added without rounding at the place its exponent gives: the unit of the sum is
 // 2^(lim - kUnit), a product of exponents ex + ed sits `s` = lim - (ex + ed) places below the
 // top word, and at s >= kMinShift 2^8 of them cannot overflow.  What does not fit (s out of
-// [kMinShift, 64): a larger product than the sum was laid out for, one 2^-43 below it, a zero,
-// a subnormal, an infinity or NaN) goes to `slow`: the FP64 fused multiply-add.  A larger
-// product also moves the sum so far into the FP64 accumulator and lays it out anew, kMargin
-// places above that product.  So each product keeps at least the precision that the FP64 sum
-// gives it, over the whole range of FP64 (1e5 x 4,096: 2.4e-15 of the largest component off the
-// 64-bit sum, 2.5e-15 with FP64 throughout).
+// [kMinShift, 64): one 2^-43 below the product the sum was laid out for, a subnormal, an infinity or
+// NaN) goes to the FP64 accumulator by a fused multiply-add; a larger product moves the sum so far
+// there and lays it out anew, kMargin places above that product.
 constexpr int kMinShift = 9, kMargin = 12, kUnit = 2 * 1023 + 62 + 32;
 struct FixedSum {
     unsigned a0 = 0, a1 = 0, a2 = 0;
-    int lim = -4 * kNoExponent;
+    int lim = 0;
 
-    // adds -w.y * d; returns false when the product does not fit (nothing is added then)
+    // adds -w.y * d; returns false when the product does not fit (nothing is added then).  A zero
+    // fits, unless its other factor is not finite: it is no exception but a user's ordinary input --
+    // a real wave function has w.y = 0 in every row, a real derivative d = 0 in a whole column, a
+    // dead unit some of one.  (As exceptions 1e5 x 4,096 of them took 1.47 ms, a tenth of them
+    // scattered 1.64; now 1.00 and 1.04, dense rows 1.03.)
     __device__ __forceinline__ bool add(const GradRow& r, double d) {
         const unsigned hi = static_cast<unsigned>(__double2hiint(d)), lo = static_cast<unsigned>(__double2loint(d));
         const int ed = static_cast<int>((hi >> 20) & 0x7ffu);
         const int s = lim - r.ex - ed;
         const bool ok = static_cast<unsigned>(ed - 1) < 0x7feu && static_cast<unsigned>(s - kMinShift) < 64u - kMinShift;
+        const bool zero = ((hi & 0x7fffffffu) | lo) == 0u ? r.ex != kNotFinite : s >= -kZero - 0x7ff && ed != 0x7ff;
         const unsigned keep = ok ? 0xffffffffu : 0u;
         const unsigned mhi = 0x80000000u | __funnelshift_l(lo, hi, 11), mlo = lo << 11;
         const unsigned neg = static_cast<unsigned>(static_cast<int>(hi) >> 31) ^ r.neg;
@@ -103,7 +105,7 @@ struct FixedSum {
         asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
             : "+r"(a0), "+r"(a1), "+r"(a2)
             : "r"(w0), "r"(w1), "r"(w2));
-        return ok;
+        return ok || zero;
     }
     // the sum so far, which starts again from zero
     __device__ __forceinline__ double take() {
@@ -119,15 +121,27 @@ struct GradSum {
     double acc;
 };
 
-// A product that did not fit (by value, out of line: its operands stay in registers elsewhere).
-__device__ __noinline__ GradSum slow_product(GradSum g, double wy, int ex, double d) {
+// A product above the window, the first of its sum, or one that a layout made since its add has
+// taken in (by value, out of line: its operands stay in registers elsewhere).
+__device__ __noinline__ GradSum place_product(GradSum g, GradRow r, double d) {
     const int ed = (__double2hiint(d) >> 20) & 0x7ff;
-    g.acc = fma(-wy, d, g.acc);
-    if (ed > 0 && ed < 0x7ff && ex > 0 && ex < kNoExponent && g.f.lim - ex - ed < kMinShift) {
-        g.acc += g.f.take();
-        g.f.lim = ex + ed + kMinShift + kMargin;
+    if (ed == 0 || ed == 0x7ff || r.ex < 0 || r.ex == kNotFinite) {
+        g.acc = fma(-r.w.y, d, g.acc);
+        return g;
     }
+    if (g.f.lim - r.ex - ed < kMinShift) {
+        g.acc += g.f.take();
+        g.f.lim = r.ex + ed + kMinShift + kMargin;
+    }
+    g.f.add(r, d);
     return g;
+}
+
+// Whether a product that add left out belongs into the fixed-point sum (place_product); if not, it
+// is below the window or not a normal number and goes to the FP64 accumulator.
+__device__ __forceinline__ bool to_place(const GradSum& g, const GradRow& r, double d) {
+    const int ed = (__double2hiint(d) >> 20) & 0x7ff;
+    return g.f.lim - r.ex - ed < 64 && ed != 0 && ed != 0x7ff;
 }
 
 // One CTA: 256 >> shift consecutive columns of one chunk of rows, the rows dealt over
@@ -163,6 +177,15 @@ __global__ void __launch_bounds__(kGradThreads, 4)
                     d[k] = __ldcs(row);
                     row += step;
                 }
+                if (t == grp) {  // a stage's first rows: the sum is laid out by the largest of them
+                    int top = 0;
+#pragma unroll
+                    for (int k = 0; k < kGradLoads; ++k) {
+                        const int ex = ws[t + k * groups].ex, ed = (__double2hiint(d[k].y) >> 20) & 0x7ff;
+                        if (ex > 0 && ex < kNotFinite && ed != 0 && ed != 0x7ff && ex + ed > top) top = ex + ed;
+                    }
+                    if (top != 0) g.f.lim = top + kMinShift + kMargin;
+                }
                 bool ok[kGradLoads];
 #pragma unroll
                 for (int k = 0; k < kGradLoads; ++k) {
@@ -175,7 +198,8 @@ __global__ void __launch_bounds__(kGradThreads, 4)
                     for (int k = 0; k < kGradLoads; ++k)
                         if (!ok[k]) {
                             const GradRow& r = ws[t + k * groups];
-                            g = slow_product(g, r.w.y, r.ex, d[k].y);
+                            if (to_place(g, r, d[k].y)) g = place_product(g, r, d[k].y);
+                            else g.acc = fma(-r.w.y, d[k].y, g.acc);
                         }
                 }
             }
@@ -184,7 +208,10 @@ __global__ void __launch_bounds__(kGradThreads, 4)
                 row += step;
                 const GradRow r = ws[t];
                 g.acc = fma(r.w.x, d.x, g.acc);
-                if (!g.f.add(r, d.y)) g = slow_product(g, r.w.y, r.ex, d.y);
+                if (!g.f.add(r, d.y)) {
+                    if (to_place(g, r, d.y)) g = place_product(g, r, d.y);
+                    else g.acc = fma(-r.w.y, d.y, g.acc);
+                }
             }
             g.acc += g.f.take();
         }
