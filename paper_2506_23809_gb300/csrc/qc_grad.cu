@@ -10,7 +10,7 @@
 // coalesced along a row): 0.97 ms for 1e5 x 4,096 at the 6.78 TB/s of a copy.  Two FP64
 // fused multiply-adds per element would take 1.38 ms (the FP64 pipe retires two per clock and
 // SM), so the real parts go through that pipe and the imaginary parts through integer
-// multiplications (FixedSum), which run beside it: 1.44 -> 1.00 ms a call, 6.6 TB/s.
+// multiplications (FixedSum), which run beside it: 1.44 -> 0.98 ms a call, 6.7 TB/s.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -65,17 +65,19 @@ __device__ __forceinline__ GradRow grad_row(double2 w) {
     return r;
 }
 
-// A sum of FP64 products in 96-bit fixed point, on the integer pipes.  A product is the top 64
-// bits of the mantissas' product (short of it by less than 3 units of its last place: 2^-60
-// relative), added without rounding at the place its exponent gives: the unit of the sum is
-// 2^(lim - kUnit), a product of exponents ex + ed sits `s` = lim - (ex + ed) places below the
-// top word, and at s >= kMinShift 2^8 of them cannot overflow.  What does not fit (s out of
-// [kMinShift, 64): one 2^-43 below the product the sum was laid out for, a subnormal, an infinity or
-// NaN) goes to the FP64 accumulator by a fused multiply-add; a larger product moves the sum so far
-// there and lays it out anew, kMargin places above that product.
-constexpr int kMinShift = 9, kMargin = 12, kUnit = 2 * 1023 + 62 + 32;
+// A sum of FP64 products in 128-bit fixed point, on the integer pipes.  A product is the top 64
+// bits of the mantissas' product (short of it by less than 3 units of its last place: 2^-61
+// relative, and exact where it fits 53 bits), added whole at the place its exponent gives: the unit
+// of the sum is 2^(lim - kUnit), a product of exponents ex + ed sits s = lim - (ex + ed) places below
+// the top word, and at s >= kMinShift 2^8 of them cannot overflow.  So in the window [kMinShift, 64)
+// of 55 binades no product loses anything to larger ones, which may have cancelled by the end (with
+// 96 bits a product 2^42 below the window's top kept 33 bits: 200 rows of which two cancel, 2^30
+// above the rest, were off by 2e-8).  A larger product moves the sum so far into the FP64
+// accumulator and lays it out anew, kMargin places above that product; one below the window, a
+// subnormal, an infinity or NaN goes to the FP64 accumulator by a fused multiply-add.
+constexpr int kMinShift = 9, kMargin = 12, kUnit = 2 * 1023 + 62 + 64;
 struct FixedSum {
-    unsigned a0 = 0, a1 = 0, a2 = 0;
+    unsigned a0 = 0, a1 = 0, a2 = 0, a3 = 0;
     int lim = 0;
 
     // adds -w.y * d; returns false when the product does not fit (nothing is added then).  A zero
@@ -94,25 +96,31 @@ struct FixedSum {
         const unsigned neg = static_cast<unsigned>(static_cast<int>(hi) >> 31) ^ r.neg;
         unsigned long long p = static_cast<unsigned long long>(mhi) * r.mhi + __umulhi(mhi, r.mlo);
         p += __umulhi(mlo, r.mhi);
-        // one's complement for a negative product: a unit of the sum short, 2^-75 of the product
+        // the one's complement of a negative product, to the last bit of the sum, and a carry into it
         const unsigned m = neg & keep;
         const unsigned pl = (static_cast<unsigned>(p) ^ neg) & keep, ph = (static_cast<unsigned>(p >> 32) ^ neg) & keep;
-        const unsigned f0 = __funnelshift_r(m, pl, s), f1 = __funnelshift_r(pl, ph, s);
+        const unsigned f0 = __funnelshift_r(m, pl, s), f1 = __funnelshift_r(pl, ph, s), f2 = __funnelshift_r(ph, m, s);
         const bool far = s >= 32;
-        // arithmetic shift of the signed product: the word above it is its sign
-        const unsigned f2 = __funnelshift_r(ph, m, s);
-        const unsigned w0 = far ? f1 : f0, w1 = far ? f2 : f1, w2 = far ? m : f2;
-        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
-            : "+r"(a0), "+r"(a1), "+r"(a2)
-            : "r"(w0), "r"(w1), "r"(w2));
+        const unsigned w0 = far ? f0 : m, w1 = far ? f1 : f0, w2 = far ? f2 : f1, w3 = far ? m : f2;
+        asm("{\n\t.reg .u32 c;\n\tadd.cc.u32 c, %8, 1;\n\t"
+            "addc.cc.u32 %0, %0, %4;\n\taddc.cc.u32 %1, %1, %5;\n\taddc.cc.u32 %2, %2, %6;\n\taddc.u32 %3, %3, %7;\n\t}"
+            : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3)
+            : "r"(w0), "r"(w1), "r"(w2), "r"(w3), "r"(m));
         return ok || zero;
     }
-    // the sum so far, which starts again from zero
+    // the sum so far; it starts again from zero, with no layout
     __device__ __forceinline__ double take() {
-        const double low = __ull2double_rn((static_cast<unsigned long long>(a1) << 32) | a0);
-        const double v = fma(static_cast<double>(static_cast<int>(a2)), 18446744073709551616.0, low);
-        a0 = a1 = a2 = 0u;
-        return v == 0.0 ? 0.0 : ldexp(v, lim - kUnit);
+        const bool neg = static_cast<int>(a3) < 0;
+        unsigned long long h = (static_cast<unsigned long long>(a3) << 32) | a2, l = (static_cast<unsigned long long>(a1) << 32) | a0;
+        if (neg) {
+            l = ~l + 1ULL;
+            h = ~h + (l == 0ULL ? 1ULL : 0ULL);
+        }
+        const double v = fma(__ull2double_rn(h), 18446744073709551616.0, __ull2double_rn(l));
+        const int e = lim - kUnit;
+        a0 = a1 = a2 = a3 = 0u;
+        lim = 0;
+        return v == 0.0 ? 0.0 : ldexp(neg ? -v : v, e);
     }
 };
 
