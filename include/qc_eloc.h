@@ -257,8 +257,9 @@ qc_status qc_eloc_timings(qc_eloc* handle, float* ms3);
  *     (the signed elements <x|H|x'> of Eq. 2 by the Slater-Condon rules, in the handle's
  *     precision), diag_out double[n_u] (<x|H|x> with e_core).  A sample with a wrong
  *     electron count gets NaN diagonal and elements and zero keys.
- *   qc_eloc_apply: E_loc(x_i) = diag_i + sum_j elems_ij psi_conn_ij / psi_i (FP64, fixed
- *     order), then the Eq. 1 reduction over the chunk into the handle's device summary and,
+ *   qc_eloc_apply: E_loc(x_i) = diag_i + sum_j elems_ij psi_conn_ij / psi_i (FP64, in an order
+ *     that P alone fixes: a sample's E_loc has the same bits in any chunk), then the Eq. 1
+ *     reduction over the chunk into the handle's device summary and,
  *     if `summary` is given (host memory, page-locked keeps it asynchronous), a copy.
  *     psi device complex128[n_u], counts int64[n_u], elems / diag as exported, psi_conn
  *     complex128[n_u * P] in the export order, eloc_out complex128[n_u].  psi(x) = 0 gives
@@ -304,7 +305,8 @@ qc_status qc_dedup(const uint64_t* raw, int64_t n_raw, int n_orb, uint64_t* keys
  *   dconj   complex128[n_u][n_par], row-major: d/d theta_p ln Psi*(n_i); NULL if g_out is
  *   w_out   complex128[n_u] or NULL
  *   g_out   double[n_par] or NULL
- * The contraction reads dconj once (HBM-bound) in a fixed summation order (deterministic).
+ * The contraction reads dconj once (HBM-bound) in a summation order fixed by n_u and n_par
+ * (deterministic; parameters taken in several calls can differ in the last bits).
  * Errors: QC_ERR_ARG (sizes, NULL, alignment: 16 bytes, counts and g_out 8), QC_ERR_OOM
  * for the handle's n_par x (<= 512) partials buffer. */
 qc_status qc_eloc_grad(qc_eloc* handle, const double* eloc, const int64_t* counts, int64_t n_u,

@@ -317,119 +317,215 @@ __device__ __forceinline__ void apply_finish(double re, double im, double2 p, do
     *eloc = out;
 }
 
-// One lane's share of the products elems[j] psi[j], j = j0, j0 + step, ... < j1: kAppUnroll
-// independent partial sums (their loads in flight together), added in a fixed order.
-constexpr int kAppUnroll = 4;
-__device__ __forceinline__ double2 apply_products(const double* __restrict__ e, const double2* __restrict__ q,
-                                                  long long j0, long long j1, long long step) {
-    double re[kAppUnroll], im[kAppUnroll];
-#pragma unroll
-    for (int k = 0; k < kAppUnroll; ++k) re[k] = im[k] = 0.0;
-    long long j = j0;
-    for (; j + (kAppUnroll - 1) * step < j1; j += kAppUnroll * step) {
-        double h[kAppUnroll];
-        double2 v[kAppUnroll];
-#pragma unroll
-        for (int k = 0; k < kAppUnroll; ++k) {
-            h[k] = __ldcs(e + j + k * step);
-            v[k] = __ldcs(q + j + k * step);
-        }
-#pragma unroll
-        for (int k = 0; k < kAppUnroll; ++k) {
-            re[k] = fma(h[k], v[k].x, re[k]);
-            im[k] = fma(h[k], v[k].y, im[k]);
-        }
-    }
-    for (; j < j1; j += step) {
-        const double h = __ldcs(e + j);
-        const double2 v = __ldcs(q + j);
-        re[0] = fma(h, v.x, re[0]);
-        im[0] = fma(h, v.y, im[0]);
-    }
-    return make_double2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
+// The sum of one sample's P products elems[j] psi[j] has one order, given by P alone, so a sample's
+// E_loc has the same bits whatever else its call holds.  Runs of `run` products are dealt to
+// `blocks` blocks in turn; a block is summed by 128 accumulators (accumulator a takes products a,
+// a + 128, .. of each of its runs, one after another) or, in long blocks, twice as many (added in
+// pairs a, a + 128); then, for each accumulator, the blocks are added by fours and the fours one after
+// another; then the accumulators by a fixed tree.  Accumulators and blocks go to lanes, warps or
+// CTAs as the call's size asks.  (A split by the threads at hand gave a chunk's last samples other
+// bits than the whole call's.)
+constexpr int kAppAcc = 128, kAppBlocks = 32, kAppFour = 4;
+struct AppOrder {
+    int P, run, blocks;
+    bool pairs;
+};
+// One block up to 8,192 products (a warp's or 128 threads' work); beyond, one per run of 2,048 (a block
+// more is two FP64 additions an accumulator, against 32 for its products) until they are as many as
+// a cluster has groups of 128 threads.  From 64 products an accumulator on, a thread's four products
+// in flight go to two accumulators, half as long a chain of additions: N=120, 200 samples 1,019 ->
+// 994 us.
+AppOrder apply_order(long long P) {
+    const int run = P <= 8192 ? 8192 : 2048;
+    const long long n = std::max<long long>(1, (P + run - 1) / run);
+    return AppOrder{static_cast<int>(P), run, static_cast<int>(std::min<long long>(n, kAppBlocks)),
+                    P >= 64LL * kAppBlocks * kAppAcc};
 }
 
-// Many samples or short connected sets: one warp per sample.  The P products are summed
-// lane-wise in FP64 (fixed lanes, fixed shuffle tree: deterministic).
-__global__ void __launch_bounds__(256) eloc_apply_kernel(const double* __restrict__ elems,
-                                                         const double* __restrict__ diag,
-                                                         const double2* __restrict__ psi_conn,
-                                                         const double2* __restrict__ psi, long long n_u,
-                                                         long long P, double2* __restrict__ eloc,
-                                                         Counters* __restrict__ ctr) {
+// Adds v to a sum, or begins it.
+__device__ __forceinline__ void add_to(double2& sum, double2 v, bool first) {
+    sum.x = first ? v.x : sum.x + v.x;
+    sum.y = first ? v.y : sum.y + v.y;
+}
+
+// Products j, j + step, .. below end, U loads in flight, to ACC accumulators in turn.  APART: the last
+// few by code of their own, so that the loop needs no predicates and fewer registers.
+template <int ACC, int U, int UNROLL, bool APART>
+__device__ __forceinline__ void add_products(const double* __restrict__ e, const double2* __restrict__ q, int j,
+                                             int step, int end, double2 (&v)[ACC]) {
+    double h[U];
+    double2 w[U];
+#pragma unroll UNROLL
+    for (; j + (APART ? (U - 1) * step : 0) < end; j += U * step) {
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (APART || j + k * step < end) {
+                h[k] = __ldcs(e + j + k * step);
+                w[k] = __ldcs(q + j + k * step);
+            }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (APART || j + k * step < end) {
+                v[k % ACC].x = fma(h[k], w[k].x, v[k % ACC].x);
+                v[k % ACC].y = fma(h[k], w[k].y, v[k % ACC].y);
+            }
+    }
+    if (APART && j < end) {
+#pragma unroll
+        for (int k = 0; k < U - 1; ++k)
+            if (j + k * step < end) {
+                h[k] = __ldcs(e + j + k * step);
+                w[k] = __ldcs(q + j + k * step);
+            }
+#pragma unroll
+        for (int k = 0; k < U - 1; ++k)
+            if (j + k * step < end) {
+                v[k % ACC].x = fma(h[k], w[k].x, v[k % ACC].x);
+                v[k % ACC].y = fma(h[k], w[k].y, v[k % ACC].y);
+            }
+    }
+}
+
+// The sum of 128 accumulators, four to a lane.
+__device__ __forceinline__ double2 add_accumulators(double2 a, double2 b, double2 c, double2 d) {
+    return make_double2(warp_sum((a.x + b.x) + (c.x + d.x)), warp_sum((a.y + b.y) + (c.y + d.y)));
+}
+
+// Many samples of one block: one warp per sample, a lane four accumulators.  A warp takes `run`
+// consecutive samples and finishes them together, a lane each: one at a time their divisions kept the
+// FP64 pipe (16 cycles an instruction of a warp, however few its lanes) longer than P = 204 products
+// do (300,000 samples 836 -> 630 us).  APART, with five CTAs an SM, from 1,024 products on (P = 2,220,
+// 20,000 samples 232 us, 258 without; P = 609 138, 119 without).
+template <bool APART>
+__global__ void __launch_bounds__(256, APART ? 5 : 4) eloc_apply_kernel(const double* __restrict__ elems,
+                                                                        const double* __restrict__ diag,
+                                                                        const double2* __restrict__ psi_conn,
+                                                                        const double2* __restrict__ psi,
+                                                                        long long n_u, int run, int P,
+                                                                        double2* __restrict__ eloc,
+                                                                        Counters* __restrict__ ctr) {
+    constexpr int U = kAppAcc / 32;
     const int lane = threadIdx.x & 31;
     const long long warps = static_cast<long long>(gridDim.x) * (blockDim.x >> 5);
-    for (long long s = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); s < n_u;
-         s += warps) {
-        const double2 t = apply_products(elems + s * P, psi_conn + s * P, lane, P, 32);
-        const double re = warp_sum(t.x), im = warp_sum(t.y);
-        if (lane == 0) apply_finish(re, im, psi[s], diag[s], eloc + s, ctr);
+    for (long long s0 = (static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * run; s0 < n_u;
+         s0 += warps * run) {
+        const int m = n_u - s0 < run ? static_cast<int>(n_u - s0) : run;
+        double2 mine = make_double2(0.0, 0.0);
+        for (int i = 0; i < m; ++i) {
+            double2 v[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) v[k] = make_double2(0.0, 0.0);
+            add_products<U, 4, APART ? 1 : 2, APART>(elems + (s0 + i) * P, psi_conn + (s0 + i) * P, lane, 32, P, v);
+            const double2 t = add_accumulators(v[0], v[1], v[2], v[3]);
+            if (lane == i) mine = t;
+        }
+        if (lane < m) apply_finish(mine.x, mine.y, psi[s0 + lane], diag[s0 + lane], eloc + s0 + lane, ctr);
     }
 }
 
-// Long connected sets: 128 threads, or a cluster of R CTAs of 512, per sample.  The stream is
-// bound by HBM and, a close second, by the FP64 pipe (24 B and two fused multiply-adds per
-// pair), so what matters is that every SM has loads in flight whatever the number of samples:
-// a chunk of a large molecule is a few hundred samples of 10^6 pairs, and a warp per sample
-// left all but 200 warps of the chip idle (N=120, 200 samples, 5.7 GB: 11.1 ms; now 0.98 ms,
-// 5.9 TB/s).  Each CTA sums a contiguous share of the sample's pairs; the CTA sums are read
-// over distributed shared memory by the first CTA in rank order, so the result is
-// deterministic and needs no workspace.
-template <int T>
-__global__ void __launch_bounds__(T) eloc_apply_wide_kernel(const double* __restrict__ elems,
-                                                            const double* __restrict__ diag,
-                                                            const double2* __restrict__ psi_conn,
-                                                            const double2* __restrict__ psi, long long P,
-                                                            double2* __restrict__ eloc, Counters* __restrict__ ctr) {
-    __shared__ double2 warp_part[T / 32];
-    __shared__ double2 cta_part;
+// Accumulator a's sum of block b (ACC = 2: accumulators a's and a + 128's).
+template <int ACC, int U, int UNROLL>
+__device__ __forceinline__ double2 block_products(const double* __restrict__ e, const double2* __restrict__ q,
+                                                  const AppOrder& o, int b, int a) {
+    double2 v[ACC];
+#pragma unroll
+    for (int k = 0; k < ACC; ++k) v[k] = make_double2(0.0, 0.0);
+    for (int c = b * o.run; c < o.P; c += o.blocks * o.run)
+        add_products<ACC, U, UNROLL, true>(e, q, c + a, kAppAcc, min(c + o.run, o.P), v);
+    if (ACC == 2) add_to(v[0], v[ACC - 1], false);
+    return v[0];
+}
+
+// Long connected sets: a thread one accumulator (PAIRS: two), 128 threads (G = 1), or a cluster of R
+// CTAs of four times 128 (G = 4), per sample.  The stream is bound by HBM and, a close second, by the
+// FP64 pipe (24 B and two fused multiply-adds per pair), so what matters is that every SM has loads
+// in flight whatever the number of samples: a chunk of a large molecule is a few hundred samples of
+// 10^6 pairs, and a warp per sample left all but 200 warps of the chip idle (N=120, 200 samples,
+// 5.7 GB: 11.1 ms; now 0.97 ms, 5.9 TB/s).  With G = 4 a CTA's groups take the four blocks of a four; the
+// fours' sums stay in shared memory and the first CTA adds all of the sample's in order, over
+// distributed shared memory.  No workspace.  G = 1 has eight CTAs an SM with eight loads a thread in
+// flight, or ten with four (kept for calls of several waves: P = 11,340, 20,000 samples 908 us, 931
+// with eight loads; 40 samples of 5,040 41 and 35 us).
+template <int G, bool PAIRS, int PER_SM>
+__global__ void __launch_bounds__(kAppAcc * G, PER_SM) eloc_apply_wide_kernel(const double* __restrict__ elems,
+                                                                      const double* __restrict__ diag,
+                                                                      const double2* __restrict__ psi_conn,
+                                                                      const double2* __restrict__ psi,
+                                                                      const AppOrder o, double2* __restrict__ eloc,
+                                                                      Counters* __restrict__ ctr) {
+    static_assert(G == kAppFour || (G == 1 && !PAIRS), "a CTA takes whole fours of blocks");
+    constexpr int kFours = kAppBlocks / kAppFour;
+    __shared__ double2 acc[kAppAcc];
+    __shared__ double2 part[G > 1 ? 2 : 1][G][kAppAcc], fours[G > 1 ? kFours : 1][kAppAcc];
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-    const unsigned R = cl.num_blocks(), r = cl.block_rank();
+    const int R = static_cast<int>(cl.num_blocks()), r = static_cast<int>(cl.block_rank());
     const long long s = blockIdx.x / R;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double2 t = apply_products(elems + s * P, psi_conn + s * P, P * r / R + threadIdx.x, P * (r + 1) / R, T);
-    const double re = warp_sum(t.x), im = warp_sum(t.y);
-    if (lane == 0) warp_part[warp] = make_double2(re, im);
-    __syncthreads();
-    double sr = 0.0, si = 0.0;
-    if (warp == 0) {
-        const double2 v = lane < T / 32 ? warp_part[lane] : make_double2(0.0, 0.0);
-        sr = warp_sum(v.x);
-        si = warp_sum(v.y);
-        if (R > 1 && lane == 0) cta_part = make_double2(sr, si);
-    }
-    if (R > 1) {
-        cl.sync();
-        if (r == 0 && threadIdx.x == 0) {
-            for (unsigned k = 1; k < R; ++k) {
-                const double2 v = *cl.map_shared_rank(&cta_part, k);
-                sr += v.x;
-                si += v.y;
+    const double* e = elems + s * o.P;
+    const double2* q = psi_conn + s * o.P;
+    const int a = threadIdx.x % kAppAcc, g = threadIdx.x / kAppAcc;
+    double2 total = make_double2(0.0, 0.0);
+    if (G == 1) {
+        double2 four = total;
+        for (int b = 0; b < o.blocks; ++b) {
+            add_to(four, block_products<1, PER_SM == 8 ? 8 : 4, PER_SM == 8 ? 1 : 2>(e, q, o, b, a), b % kAppFour == 0);
+            if (b % kAppFour == kAppFour - 1 || b == o.blocks - 1) add_to(total, four, b < kAppFour);
+        }
+    } else {
+        const int n = (o.blocks + kAppFour - 1) / kAppFour, own = (n + R - 1) / R;  // fours, and of one CTA
+        for (int f = r * own; f < (r + 1) * own && f < n; ++f) {
+            if (f * kAppFour + g < o.blocks) part[f & 1][g][a] = block_products<PAIRS ? 2 : 1, 4, 1>(e, q, o, f * kAppFour + g, a);
+            __syncthreads();  // (the other half of part is read before the next one)
+            if (g == 0) {
+                double2 four = part[f & 1][0][a];
+#pragma unroll
+                for (int k = 1; k < kAppFour; ++k)
+                    if (f * kAppFour + k < o.blocks) add_to(four, part[f & 1][k][a], false);
+                fours[f - r * own][a] = four;
             }
         }
-        cl.sync();  // the other CTAs' sums stay in place until the first CTA has read them
+        if (R > 1) cl.sync();
+        if (r == 0 && g == 0)
+            for (int f = 0; f < n; ++f) {
+                const double2 v = R > 1 ? cl.map_shared_rank(&fours[0][0], f / own)[f % own * kAppAcc + a] : fours[f][a];
+                add_to(total, v, f == 0);
+            }
+        if (R > 1) cl.sync();  // the other CTAs' sums stay in place until the first CTA has read them
     }
-    if (r == 0 && threadIdx.x == 0) apply_finish(sr, si, psi[s], diag[s], eloc + s, ctr);
+    if (r != 0) return;
+    if (g == 0) acc[a] = total;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const double2 t = add_accumulators(acc[a], acc[a + 32], acc[a + 64], acc[a + 96]);
+        if (a == 0) apply_finish(t.x, t.y, psi[s], diag[s], eloc + s, ctr);
+    }
 }
 
-// Threads per sample: two full waves of the chip's threads over the samples; 32 (a warp), 128, or
-// R x 512 with R up to the portable cluster size.  With many samples a CTA's fixed cost (block
-// sum, launch) pays only for long sums (10,000 samples, P = 2,220: 140 us with a warp, 167 us with
-// 128 threads; P = 5,040: 277 against 311 us; P = 7,875: 381 against 361; P = 25,137: 1,102 against 983);
-// with few, idle SMs cost more (300 samples, P = 25,137: 270 us with a warp, 106 us).
-int apply_threads(long long n_u, long long P, int sm_count) {
-    const long long cap = n_u >= 8LL * sm_count ? P / 160 : P / 8;
-    const long long want = std::min(2LL * 2048 * sm_count / n_u, cap);
-    if (want <= 48) return 32;
-    if (want < 256 || (want < 512 && P < 32768)) return 128;
-    int t = 512;
-    while (t < 8 * 512 && want >= 2 * t) t *= 2;
-    return t;
+// Threads per sample: 32 (a warp), 128, or R x 512 with R up to the portable cluster size and the fours
+// of blocks.  One block: 128 while they are resident together, then a warp (P = 2,220, 1,300 samples
+// 48 us against 54, 10,000 148 against 139; from 6,144 products 128 always: P = 7,875, 5,000 samples 201
+// against 224).  Above 16,384 products 512 R by how the samples fill waves of three CTAs an SM: few
+// take the whole cluster, up to three an SM one CTA each (300 samples: P = 25,137 65 us, 79 with R = 4;
+// 599,360 682, 730 with R = 8), then 128 threads or R = 4, whose waves are finer (500 samples: P = 25,137
+// 96 us, 109 with R = 1; 294,750 629, 816 with R = 1), and many again one CTA each (P = 25,137, 10,000
+// samples 990 us, 1,040 with 128 threads).
+int apply_threads(long long n_u, const AppOrder& o, int sm_count) {
+    const long long sm = sm_count;
+    if (o.blocks == 1) return n_u <= 9 * sm || o.P >= 6144 ? 128 : 32;
+    if (o.P <= 16384 && n_u > 2 * sm) return 128;
+    int R;
+    if (o.P < 65536)
+        R = n_u <= sm * 4 / 5 ? 4 : n_u <= 3 * sm || n_u > 8 * sm ? 1 : 0;
+    else
+        R = n_u <= sm * 8 / 5 ? 8 : n_u <= 3 * sm || n_u > 8 * sm ? 1 : 4;
+    if (R == 0) return 128;
+    const int fours = (o.blocks + kAppFour - 1) / kAppFour;
+    while (R > fours) R /= 2;
+    return 512 * R;
 }
 
-template <int T>
+template <int G, bool PAIRS, int PER_SM>
 cudaError_t launch_apply_wide(const double* elems, const double* diag, const double2* conn, const double2* psi,
-                              long long n_u, long long P, double2* eloc, Counters* ctr, int R, cudaStream_t s) {
+                              long long n_u, const AppOrder& o, double2* eloc, Counters* ctr, int R, cudaStream_t s) {
     // a grid holds fewer than 2^31 blocks: longer chunks go out in several launches
     const long long most = 0x7fffffffLL / R;
     cudaError_t e = cudaSuccess;
@@ -437,7 +533,7 @@ cudaError_t launch_apply_wide(const double* elems, const double* diag, const dou
         const long long n = std::min(most, n_u - lo);
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(static_cast<unsigned>(n * R));
-        cfg.blockDim = dim3(T);
+        cfg.blockDim = dim3(kAppAcc * G);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -446,7 +542,7 @@ cudaError_t launch_apply_wide(const double* elems, const double* diag, const dou
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, eloc_apply_wide_kernel<T>, elems + lo * P, diag + lo, conn + lo * P, psi + lo, P,
+        e = cudaLaunchKernelEx(&cfg, eloc_apply_wide_kernel<G, PAIRS, PER_SM>, elems + lo * o.P, diag + lo, conn + lo * o.P, psi + lo, o,
                                eloc + lo, ctr);
     }
     return e;
@@ -542,15 +638,26 @@ extern "C" qc_status qc_eloc_apply(qc_eloc* H, const double* psi, const int64_t*
         const double2* conn = reinterpret_cast<const double2*>(psi_conn);
         const double2* p2 = reinterpret_cast<const double2*>(psi);
         double2* el = reinterpret_cast<double2*>(eloc_out);
-        const int t = qc::apply_threads(n_u, H->sp.pairs, H->sm_count);
+        const qc::AppOrder o = qc::apply_order(H->sp.pairs);
+        const int t = qc::apply_threads(n_u, o, H->sm_count);
         if (t >= 512) {
-            e = qc::launch_apply_wide<512>(elems, diag, conn, p2, n_u, H->sp.pairs, el, H->d_ctr, t / 512, s);
+            // two CTAs an SM with pairs (N=120, 200 samples 992 us, 1,043 with three) but where three
+            // hold every CTA at once (40 samples 309, 346 with two), and three without pairs but where
+            // two fill their second wave better
+            const long long ctas = n_u * (t / 512), sm = H->sm_count;
+            const auto f = o.pairs ? ctas > 2 * sm && ctas <= 3 * sm ? qc::launch_apply_wide<4, true, 3>
+                                                                     : qc::launch_apply_wide<4, true, 2>
+                           : ctas > 3 * sm && ctas <= 4 * sm ? qc::launch_apply_wide<4, false, 2>
+                                                             : qc::launch_apply_wide<4, false, 3>;
+            e = f(elems, diag, conn, p2, n_u, o, el, H->d_ctr, t / 512, s);
         } else if (t == 128) {
-            e = qc::launch_apply_wide<128>(elems, diag, conn, p2, n_u, H->sp.pairs, el, H->d_ctr, 1, s);
+            const auto f = n_u <= 5LL * H->sm_count ? qc::launch_apply_wide<1, false, 8> : qc::launch_apply_wide<1, false, 10>;
+            e = f(elems, diag, conn, p2, n_u, o, el, H->d_ctr, 1, s);
         } else {
-            const long long blocks = std::min<long long>((n_u + 7) / 8, static_cast<long long>(H->sm_count) * 16);
-            qc::eloc_apply_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(elems, diag, conn, p2, n_u,
-                                                                              H->sp.pairs, el, H->d_ctr);
+            const long long warps = std::min<long long>(n_u, static_cast<long long>(H->sm_count) * 128);
+            const int run = static_cast<int>(std::min<long long>(32, (n_u + warps - 1) / warps));
+            const auto f = o.P < 1024 ? qc::eloc_apply_kernel<false> : qc::eloc_apply_kernel<true>;
+            f<<<static_cast<unsigned>((warps + 7) / 8), 256, 0, s>>>(elems, diag, conn, p2, n_u, run, o.P, el, H->d_ctr);
             e = cudaGetLastError();
         }
     }
