@@ -14,20 +14,24 @@
 //   KM merge    runs merged in pairs until one is left (the run lengths and the number of
 //               passes that do something follow the device's count of distinct keys)
 //   KE emit     the sorted keys with their counts, looked up in the hash table
-// A stream with too many distinct keys for the hash table (a probe sequence longer than
-// kProbeMax ends the counting), or a short one, is sorted whole instead by the same KT and KM,
+// A stream with too many distinct keys for the hash table (by a sample of it taken while the table is
+// cleared, KS; or else a probe sequence longer than kProbeMax ends the counting), or a short one, is
+// sorted whole instead by the same KT and KM,
 // and its runs counted:
 //   KH heads    heads of runs per tile; their prefix sum; KR runs: the head keys and their
 //               positions; KC: multiplicities as differences of positions
-// Every kernel of both ways is launched; the device's flag decides which of them do anything.
+// Every kernel of both ways is launched; the device's flag decides which of them do anything.  KA and KM
+// are launched early (wait_previous): KA clears its shared memory while the global table is cleared,
+// and the merge passes that a stream does not need follow each other closely, which pays for KS.
 //
 // Keys of up to 64 orbitals are sorted as one word.  Traffic: 16 B per raw key, then 16 (or 32)
-// B per distinct key and merge pass, in place of 48 B per raw key and 8-bit digit: N=52, 10^7 raw
-// keys of 10^5 distinct: 1.02 ms with a radix sort of the whole stream, now 0.20 ms (counting 78 us,
-// listing 10, tiles 16, six merges 48, the rest launches and the clearing); of 4*10^5 distinct
-// 1.05 -> 0.26; N=120 1.92 -> 0.22.  Sorted whole: 131,000 raw keys 0.36 -> 0.08 ms; 10^7 raw keys of
-// 5*10^6 distinct 1.15 -> 1.11 ms (0.14 of them the counting that ends early); N=120, 4*10^6 of
-// 3*10^6 distinct 1.22 -> 0.79.
+// B per distinct key and merge pass, in place of 48 B per raw key and 8-bit digit of a radix sort of
+// the whole stream.  10^7 raw keys at N=52: 1.02 ms with that sort (this stream), now 0.18 (counting
+// 78 us, listing 10, tiles 16, six merges 48, the rest launches and the clearing); of 5*10^5 distinct
+// 1.40 -> 0.36.  Sorted whole: 10^5 raw keys 0.42 -> 0.07 ms; 10^7 of 5*10^6 distinct 1.87 -> 0.96, and at
+// N=28, four digits, 1.19 -> 0.96; 3*10^6 of 3*10^6 at N=28 0.41 -> 0.31 (0.49 when the counting had to
+// fail first).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -49,7 +53,7 @@ constexpr int kTile = kSortThreads * kSortItems;  // keys of a tile
 // than the merge passes it saves (131,072 raw keys: 84 us whole, 108 us counted).
 constexpr long long kCountMinRaw = 1 << 19;
 constexpr unsigned kMaxSlots = 1u << 21;    // hash table: 24 MB, L2-resident
-constexpr unsigned kProbeMax = 16;          // reached near 0.4 of the slots filled
+constexpr unsigned kProbeMax = 64;          // reached near 0.45 of the slots filled
 constexpr int kCountThreads = 1024;
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
@@ -125,11 +129,16 @@ __device__ __forceinline__ bool slot_holds(unsigned long long e, const ulonglong
                                            unsigned long long h) {
     return (e >> 32) == (h >> 32) && K::of(raw[static_cast<unsigned>(e) - 1u]).same(k);
 }
-template <typename K>
+// DIRECT: every key is its own slot number (no more orbitals than slot bits), so the table never fills.
+template <bool DIRECT, typename K>
+__device__ __forceinline__ unsigned first_slot(const K& k, unsigned long long h, unsigned mask) {
+    return (DIRECT ? static_cast<unsigned>(k.wide().x) : static_cast<unsigned>(h >> 13)) & mask;
+}
+template <bool DIRECT, typename K>
 __device__ __forceinline__ void count_global(const ulonglong2* __restrict__ raw, const K& k, unsigned i, unsigned c,
                                              unsigned long long h, unsigned long long* slot, unsigned* count,
                                              unsigned mask, Ctrl* ctrl) {
-    unsigned s = static_cast<unsigned>(h >> 13) & mask;
+    unsigned s = first_slot<DIRECT>(k, h, mask);
     for (unsigned it = 0; it < kProbeMax; ++it) {
         unsigned long long e = __ldcg(slot + s);
         if (e == 0ULL) e = atomicCAS(slot + s, 0ULL, (h >> 32 << 32) | (i + 1u));
@@ -157,8 +166,8 @@ struct CountTable {
     static constexpr size_t bytes = slots * (sizeof(K) + 12) + kCountThreads / 32 * queue * 4;
 };
 
-template <typename K>
-__global__ void __launch_bounds__(kCountThreads, 1) dedup_count_kernel(const ulonglong2* __restrict__ raw, long long n,
+template <bool DIRECT, typename K>
+__global__ void __launch_bounds__(kCountThreads, 1) dedup_count_kernel(const ulonglong2* raw, long long n,
                                                                       ulonglong2 high, unsigned long long* slot,
                                                                       unsigned* count, unsigned mask, Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -170,14 +179,15 @@ __global__ void __launch_bounds__(kCountThreads, 1) dedup_count_kernel(const ulo
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned* queue = pos + S + warp * CountTable<K>::queue;
     for (int t = threadIdx.x; t < S; t += kCountThreads) tag[t] = cnt[t] = 0u;
-    __syncthreads();
+    qc::wait_previous();
+    if (__syncthreads_or(__ldcg(&ctrl->full) != 0u)) return;  // too many distinct keys
     bool bad = false;
     int qn = 0;
     auto flush = [&](int m) {  // the first m queued raw positions to the global table
         if (lane < m) {
             const unsigned i = queue[lane];
             const K k = K::of(raw[i]);
-            count_global(raw, k, i, 1u, key_hash(k), slot, count, mask, ctrl);
+            count_global<DIRECT>(raw, k, i, 1u, key_hash(k), slot, count, mask, ctrl);
         }
         __syncwarp();
         const unsigned rest = lane < qn - m ? queue[m + lane] : 0u;
@@ -239,7 +249,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) dedup_count_kernel(const ulo
     __syncthreads();
     for (int t = threadIdx.x; t < S; t += kCountThreads)
         if (tag[t] >= 2u)
-            count_global(raw, keys[t], pos[t], cnt[t], key_hash(keys[t]), slot, count, mask, ctrl);
+            count_global<DIRECT>(raw, keys[t], pos[t], cnt[t], key_hash(keys[t]), slot, count, mask, ctrl);
 }
 
 // KL: the distinct keys into `list`, in any order (they are sorted next and are distinct).  (Listing
@@ -405,7 +415,7 @@ __global__ void __launch_bounds__(kSortThreads) dedup_tile_kernel(const ulonglon
 // 32 lanes of a warp: each step cuts the range to a 33rd, so a run of 10^6 keys takes four
 // dependent loads instead of twenty.
 template <typename K>
-__device__ __forceinline__ long long merge_split_warp(const K* __restrict__ a, long long na, const K* __restrict__ b,
+__device__ __forceinline__ long long merge_split_warp(const K* a, long long na, const K* b,
                                                       long long nb, long long d, int lane) {
     long long lo = d > nb ? d - nb : 0, hi = d < na ? d : na;  // the answer lies in [lo, hi]
     while (lo < hi) {
@@ -433,9 +443,13 @@ __global__ void __launch_bounds__(kSortThreads) dedup_merge_kernel(K* A, K* B, K
     __shared__ K tile[kTilePadded];
     __shared__ long long split[2];
     const Tile<K> sh{tile, 0};
+    qc::wait_previous();
     const bool whole = sort_whole<K>(ctrl, n);
     const long long m = whole ? n : static_cast<long long>(ctrl->m);
-    if (run >= m) return;
+    if (run >= m) {  // (a pass that merges lets the next one start by ending: earlier, 10^7 keys take 14% longer)
+        qc::let_next_start();
+        return;
+    }
     K* other = whole ? B : half;
     const K* in = odd ? other : A;
     K* out = odd ? A : other;
@@ -476,7 +490,7 @@ __device__ __forceinline__ const K* sorted_in(const K* A, const K* B, long long 
 }
 
 // KE: the distinct keys with their counts.
-template <typename K>
+template <bool DIRECT, typename K>
 __global__ void __launch_bounds__(256) dedup_emit_kernel(const ulonglong2* __restrict__ raw, long long n,
                                                          const K* __restrict__ A, const K* __restrict__ half,
                                                          const unsigned long long* __restrict__ slot,
@@ -491,7 +505,7 @@ __global__ void __launch_bounds__(256) dedup_emit_kernel(const ulonglong2* __res
          j += static_cast<long long>(gridDim.x) * blockDim.x) {
         const K k = sorted[j];
         const unsigned long long h = key_hash(k);
-        unsigned s = static_cast<unsigned>(h >> 13) & mask;
+        unsigned s = first_slot<DIRECT>(k, h, mask);
         for (unsigned it = 0; it < kProbeMax; ++it) {  // every listed key was placed within kProbeMax
             const unsigned long long e = slot[s];
             if (e == 0ULL || slot_holds(e, raw, k, h)) break;
@@ -674,11 +688,75 @@ __global__ void __launch_bounds__(256) dedup_counts_kernel(const long long* __re
         counts_out[j] = heads[j + 1] - heads[j];
 }
 
-__global__ void dedup_start_kernel(Ctrl* ctrl, unsigned full) {
-    *ctrl = Ctrl{0u, full, 0u, 0u};
+// The stream is sorted whole from the start.
+__global__ void dedup_whole_kernel(Ctrl* ctrl) { *ctrl = Ctrl{0u, 1u, 0u, 0u}; }
+
+// KS: clears the hash table (all clusters but the first) and judges by a sample (the first) whether the
+// stream has too many distinct keys for it.  kSample raw keys, one from each of as many equal parts
+// of the stream, are put in a table of 32-bit hashes spread over the cluster; c of them find their
+// hash there.  A stream in which two random places agree with probability 1/N2 has c near
+// kSample^2 / (2 N2), and at least n N2 / (n + N2) distinct keys (Cauchy-Schwarz on the
+// multiplicities).  With c taken two standard deviations high, too many by that bound are too many
+// indeed, and the counting, which would end half-way after some 100 us, is left out (3*10^6 raw keys of
+// 1.5*10^6 distinct at N=28: 444 -> 301 us; at N=20, of 8*10^5 and counted in slots of their own, 410 ->
+// 223).  By one CTA the sample took 24 us, most of it waiting for 16,384 scattered sectors; a
+// cluster's is done soon after the clearing.
+constexpr int kSample = 1 << 14, kSampleCluster = 8, kSampleSlots = 4096;  // slots of one CTA
+template <typename K>
+__global__ void __cluster_dims__(kSampleCluster, 1, 1) __launch_bounds__(1024)
+    dedup_start_kernel(const ulonglong2* __restrict__ raw, long long n, uint4* __restrict__ table, long long words,
+                       unsigned slots, bool direct, Ctrl* ctrl) {
+    __shared__ __align__(16) unsigned seen[kSampleSlots];
+    __shared__ int found;
+    qc::let_next_start();
+    const bool sampler = blockIdx.x < kSampleCluster && !direct;
+    if (!sampler) {
+        const long long first = direct ? 0 : kSampleCluster;
+        for (long long i = (blockIdx.x - first) * 1024 + threadIdx.x; i < words; i += (gridDim.x - first) * 1024)
+            table[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (blockIdx.x == 0 && threadIdx.x == 0) *ctrl = Ctrl{0u, 0u, 0u, 0u};
+        return;
+    }
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    constexpr int kOwn = kSample / (1024 * kSampleCluster);
+    const unsigned part = static_cast<unsigned>(n / kSample);
+    ulonglong2 r[kOwn];
+#pragma unroll
+    for (int k = 0; k < kOwn; ++k) {
+        const unsigned t = (blockIdx.x * kOwn + k) * 1024u + threadIdx.x;
+        const unsigned in = __umulhi((t * 0x9E3779B1u) ^ (t << 19), part);  // any place of part t
+        r[k] = raw[static_cast<long long>(t) * n / kSample + in];
+    }
+    reinterpret_cast<uint4*>(seen)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+    static_assert(kSampleSlots == 4 * 1024, "cleared by one store a thread");
+    if (threadIdx.x == 0) found = 0;
+    cl.sync();
+    int c = 0;
+#pragma unroll
+    for (int k = 0; k < kOwn; ++k) {
+        const unsigned long long h = key_hash(K::of(r[k]));
+        const unsigned mine = static_cast<unsigned>(h >> 32) | 1u;
+        unsigned* at = cl.map_shared_rank(seen, static_cast<unsigned>(h >> 16) % kSampleCluster);
+        unsigned s = static_cast<unsigned>(h) % kSampleSlots;
+        for (int it = 0; it < kSampleSlots; ++it) {
+            const unsigned old = atomicCAS(at + s, 0u, mine);
+            if (old == mine) ++c;
+            if (old == 0u || old == mine) break;
+            s = (s + 1u) % kSampleSlots;
+        }
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c != 0) atomicAdd(cl.map_shared_rank(&found, 0), c);
+    cl.sync();  // (the CTAs' tables and rank 0's count are touched no more)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const float all = static_cast<float>(found), high = all + 2.0f * sqrtf(all) + 2.0f;
+        const float n2 = 0.5f * kSample * static_cast<float>(kSample) / high, fn = static_cast<float>(n);
+        const bool many = fn * n2 / (fn + n2) > 0.45f * static_cast<float>(slots);
+        *ctrl = Ctrl{0u, many ? 1u : 0u, 0u, 0u};
+    }
 }
 
-template <typename K>
+template <bool DIRECT, typename K>
 cudaError_t dedup(const ulonglong2* raw, long long n, ulonglong2 high, ulonglong2* keys_out, long long* counts_out,
                   long long* n_unique, unsigned char* W, const Layout& L, bool count, int sms, cudaStream_t s) {
     K* A = reinterpret_cast<K*>(W + L.bufA);
@@ -693,18 +771,24 @@ cudaError_t dedup(const ulonglong2* raw, long long n, ulonglong2 high, ulonglong
     const unsigned mask = L.slots - 1u;
     const long long tiles = (n + kTile - 1) / kTile;
     const unsigned grid = static_cast<unsigned>(std::min<long long>(tiles, 8LL * sms));
-    dedup_start_kernel<<<1, 1, 0, s>>>(ctrl, count ? 0u : 1u);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (!count) {
+        dedup_whole_kernel<<<1, 1, 0, s>>>(ctrl);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess && count) {
         constexpr size_t smem = CountTable<K>::bytes;
-        e = cudaMemsetAsync(slot, 0, static_cast<size_t>(L.slots) * 12, s);
+        // a CTA an SM, in whole clusters: the count's CTAs start beside them
+        const unsigned clusters = static_cast<unsigned>(std::max(2, sms / kSampleCluster));
+        dedup_start_kernel<K><<<clusters * kSampleCluster, 1024, 0, s>>>(
+            raw, n, reinterpret_cast<uint4*>(slot), static_cast<long long>(L.slots) * 12 / 16, L.slots, DIRECT, ctrl);
+        e = cudaGetLastError();
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(dedup_count_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(dedup_count_kernel<DIRECT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      static_cast<int>(smem));
         if (e == cudaSuccess) {
-            dedup_count_kernel<K><<<static_cast<unsigned>(sms), kCountThreads, smem, s>>>(raw, n, high, slot, counts,
-                                                                                         mask, ctrl);
-            e = cudaGetLastError();
+            e = qc::launch_early(dedup_count_kernel<DIRECT, K>, dim3(static_cast<unsigned>(sms)), dim3(kCountThreads), smem, s,
+                                 true, raw, n, high, slot, counts, mask, ctrl);
         }
         if (e == cudaSuccess) {
             dedup_list_kernel<K><<<L.slots / (1024 * kListSlots), 1024, 0, s>>>(raw, slot, A, ctrl);
@@ -717,12 +801,11 @@ cudaError_t dedup(const ulonglong2* raw, long long n, ulonglong2 high, ulonglong
     }
     bool odd = false;
     for (long long run = kTile; run < n && e == cudaSuccess; run *= 2) {
-        dedup_merge_kernel<K><<<grid, kSortThreads, 0, s>>>(A, B, half, odd, n, run, ctrl);
-        e = cudaGetLastError();
+        e = qc::launch_early(dedup_merge_kernel<K>, dim3(grid), dim3(kSortThreads), 0, s, true, A, B, half, odd, n, run, ctrl);
         odd = !odd;
     }
     if (e == cudaSuccess && count) {
-        dedup_emit_kernel<K><<<4 * sms, 256, 0, s>>>(raw, n, A, half, slot, counts, mask, keys_out, counts_out,
+        dedup_emit_kernel<DIRECT, K><<<4 * sms, 256, 0, s>>>(raw, n, A, half, slot, counts, mask, keys_out, counts_out,
                                                     n_unique, ctrl);
         e = cudaGetLastError();
     }
@@ -807,8 +890,9 @@ extern "C" qc_status qc_dedup(const uint64_t* raw, int64_t n_raw, int n_orb, uin
     ulonglong2* ko = reinterpret_cast<ulonglong2*>(keys_out);
     long long* co = reinterpret_cast<long long*>(counts_out);
     long long* nu = reinterpret_cast<long long*>(n_unique);
-    e = n_orb <= 64 ? dedup<Key1>(r, n, high, ko, co, nu, W, L, count, sms, s)
-                    : dedup<Key2>(r, n, high, ko, co, nu, W, L, count, sms, s);
+    e = n_orb > 64 ? dedup<false, Key2>(r, n, high, ko, co, nu, W, L, count, sms, s)
+        : n_orb <= 31 && (1u << n_orb) <= L.slots ? dedup<true, Key1>(r, n, high, ko, co, nu, W, L, count, sms, s)
+                                                  : dedup<false, Key1>(r, n, high, ko, co, nu, W, L, count, sms, s);
     if (e != cudaSuccess) return dfail(QC_ERR_CUDA, cudaGetErrorString(e));
     return QC_OK;
 }
