@@ -651,7 +651,7 @@ qc_status qc_eloc_eval(qc_eloc* H, const uint64_t* samples, const int64_t* count
             clear.add(pa, 2 * a256(static_cast<size_t>(nt) * 4));
         }
     }
-    QC_CHK(qc::launch_clear(clear, s), "clear launch");
+    QC_CHK(qc::launch_clear(clear, H->sm_count, s), "clear launch");
     QC_CHK(qc::launch_build_table(tp, H->n_orb, H->na, H->nb, H->d_T, H->d_slots, H->d_filter, aset, bset,
                                   H->d_ctr, s, jkey, jlen, true),
            "build_table launch");

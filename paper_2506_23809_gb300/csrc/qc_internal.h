@@ -270,7 +270,7 @@ cudaError_t launch_build_table(const TableParams& tp, int n_orb, int na, int nb,
                                uint32_t* filter, unsigned long long* aset,
                                unsigned long long* bset, Counters* ctr, cudaStream_t s,
                                unsigned* jkey = nullptr, unsigned* jlen = nullptr, bool early = false);
-cudaError_t launch_clear(const ClearList& list, cudaStream_t s);
+cudaError_t launch_clear(const ClearList& list, int sm_count, cudaStream_t s);
 cudaError_t launch_eloc_main(const SysParams& sp, const TableParams& tp, const EvalParams& ep,
                              const LaunchCfg& cfg, cudaStream_t s);
 // the same kernels with the hit lists and work counters compiled in (qc_kernels_diag.cu)
@@ -320,7 +320,7 @@ cudaError_t launch_join_batch(const MolParams* mols, const unsigned* slot_base, 
                               unsigned* jlen, unsigned* jstart, ulonglong2* gent, cudaStream_t s,
                               const unsigned* row_base = nullptr, unsigned* order = nullptr,
                               unsigned* pa = nullptr, unsigned* pb = nullptr);
-// in-place exclusive prefix sum of n u32 (qc_dedup.cu); sums: (n / 4096 + 2) u32 of scratch
+// exclusive prefix sum of n u32, in place or into another array (qc_dedup.cu); sums: (n / 4096 + 2) u32 of scratch
 cudaError_t exclusive_scan_u32(const unsigned* in, unsigned* out, long long n, unsigned* sums, cudaStream_t s);
 // message returned by qc_eloc_last_error(NULL) on this thread (qc_api.cu)
 void set_handleless_error(const std::string& msg);

@@ -145,12 +145,13 @@ __global__ void __launch_bounds__(256) clear_kernel(const __grid_constant__ Clea
 // ------------------------------------------------------------------------------------
 // host launchers
 // ------------------------------------------------------------------------------------
-cudaError_t launch_clear(const ClearList& list, cudaStream_t s) {
+cudaError_t launch_clear(const ClearList& list, int sm_count, cudaStream_t s) {
     size_t most = 0;
     for (int k = 0; k < list.n; ++k) most = list.bytes[k] > most ? list.bytes[k] : most;
     // up to two 16-byte stores a thread and range, at most eight CTAs an SM
+    const size_t cap = static_cast<size_t>(sm_count) * 8;
     size_t blocks = (most / 16 + 511) / 512;
-    blocks = blocks < 1 ? 1 : blocks > 152 * 8 ? 152 * 8 : blocks;
+    blocks = blocks < 1 ? 1 : blocks > cap ? cap : blocks;
     clear_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(list);
     return cudaGetLastError();
 }
