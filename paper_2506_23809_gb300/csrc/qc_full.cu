@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(T, 1280 / T) eloc_export_kernel(const __grid_c
         }
         __syncthreads();
         if (item >= items) break;
+        if (out.keys == nullptr && out.elems == nullptr) continue;  // the diagonal alone
         const long long s = static_cast<long long>(item / C);
         const long long v0 = (static_cast<long long>(item) - s * C) * Q;
         const long long p0 = export_position(sp, v0), p1 = export_position(sp, v0 + Q) < P ? export_position(sp, v0 + Q) : P;
@@ -604,6 +605,8 @@ extern "C" qc_status qc_eloc_export(qc_eloc* H, const uint64_t* samples, int64_t
     const long long V = H->sp.pairs + (qc::export_single_weight(H->sp) - 1) * (H->sp.nsa + H->sp.nsb);
     long long C = std::max<long long>(1, (V + qc::kExpItemPairs / 2) / qc::kExpItemPairs);
     while (n_u * C < 2 * resident && V / (2 * C) >= 1024) C *= 2;
+    if (!keys_out && !elems_out) C = 1;  // the diagonal alone (N=40, 10 electrons, 20,000 samples:
+                                         // 193 us when every pair was walked for it, 48)
     const long long Q = (V + C - 1) / C;
     const long long blocks = std::min<long long>(n_u * C, resident);
     unsigned long long* cursor = &H->d_ctr->next;  // the handle's counters are free between evaluations
