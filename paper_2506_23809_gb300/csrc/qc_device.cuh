@@ -988,7 +988,8 @@ __device__ __forceinline__ float2 inv_psi32(double2 p) {
 // K2: the local-energy kernel
 // ------------------------------------------------------------------------------------
 // The kernel's speed depends on its code's size: 24 warps at different places of it make 60% of the
-// instruction cache's requests, 8% of them misses (ncu, N=52).  So its loops are not unrolled
+// requests that the instruction cache can take, 4.7% of them misses, and wait for instructions 0.73
+// warps an issue (ncu, N=52; 1.56 when the loops were unrolled).  So its loops are not unrolled
 // (`#pragma unroll 1`: the compiler's fourfold copies of loops that run a few times), and what
 // rarely runs is out of line: N=52 2.58 -> 2.47 ms a step, N=76 11.67 -> 10.98, N=40 2.61 -> 2.55.
 // One warp per sample (persistent grid).  The five excitation classes are walked as

@@ -442,7 +442,7 @@ __device__ __forceinline__ double2 block_products(const double* __restrict__ e, 
 // FP64 pipe (24 B and two fused multiply-adds per pair), so what matters is that every SM has loads
 // in flight whatever the number of samples: a chunk of a large molecule is a few hundred samples of
 // 10^6 pairs, and a warp per sample left all but 200 warps of the chip idle (N=120, 200 samples,
-// 5.7 GB: 11.1 ms; now 0.97 ms, 5.9 TB/s).  With G = 4 a CTA's groups take the four blocks of a four; the
+// 5.7 GB: 11.1 ms; now 0.95 ms, 6.0 TB/s).  With G = 4 a CTA's groups take the four blocks of a four; the
 // fours' sums stay in shared memory and the first CTA adds all of the sample's in order, over
 // distributed shared memory.  No workspace.  G = 1 has eight CTAs an SM with eight loads a thread in
 // flight, or ten with four (kept for calls of several waves: P = 11,340, 20,000 samples 908 us, 931
